@@ -41,21 +41,13 @@ struct Rec3 {
   uint32_t sgrid;
   V* q(int j) { return Q[((j % 3) + 3) % 3]; }
 
-  int apply_dot(const V* x, V* y, int* np) {
-    if (s->fast.ok) return apply_fast(s, x, y, W->st, W->partial, np);
-    ED_TRY(apply_h(s, x, y, W->st));
-    k_dot<V><<<W->grid, kRedThreads, 0, W->st>>>(x, y, W->n, W->partial);
-    ED_LAUNCH_CHECK();
-    *np = (int)W->grid;
-    return ED_OK;
-  }
   int init() {  // q_0 already in Q[0]
     return dot_to(*W, (const V*)q(0), (const V*)q(0), OP_SIGMA0, 0);
   }
   int step(int j, double thr, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr) {
     int np = 0;
     if (e0) ED_TRY_CUDA(cudaEventRecord(e0, W->st));
-    ED_TRY(apply_dot(q(j), Y, &np));
+    ED_TRY(apply_dot<V>(s, *W, q(j), Y, &np));
     if (e1) ED_TRY_CUDA(cudaEventRecord(e1, W->st));
     k_finish<<<1, kRedThreads, 0, W->st>>>(W->partial, np, OP_ALPHA_Q, j, W->c, 0.0);
     k_lz_step<V><<<sgrid, kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,

@@ -10,74 +10,14 @@
 #include <cstring>
 #include <vector>
 
+#include "cgs_tile.h"
 #include "ed_internal.h"
 #include "tri_common.h"
-#include "vec16.h"
+#include "vec_ops.h"
 
 namespace ed {
 
 namespace {
-
-constexpr int kRedThreads = 256;
-
-// ------------------------------------------------ element-level helpers
-__device__ __forceinline__ void dmac(double& a, double x, double y) { a = fma(x, y, a); }
-__device__ __forceinline__ void dmac(float2& a, float2 x, float2 y) { df_mac(a, x, y); }
-__device__ __forceinline__ void dmac(float2& a, float x, float y) { df_mac1(a, make_float2(x, 0.f), y); }
-
-__device__ __forceinline__ double to_d(double a) { return a; }
-__device__ __forceinline__ double to_d(float2 a) { return (double)a.x + (double)a.y; }
-
-__device__ __forceinline__ double add_acc(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 add_acc(float2 a, float2 b) { return df_add(a, b); }
-
-__device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ float2 shfl_x(float2 v, int o) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-
-template <class A>
-__device__ __forceinline__ A block_reduce(A v, A* sh) {
-  for (int o = 16; o > 0; o >>= 1) v = add_acc(v, shfl_x(v, o));
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  int nw = blockDim.x >> 5;
-  if (w == 0) {
-    v = (lane < nw) ? sh[lane] : A{};
-    for (int o = 16; o > 0; o >>= 1) v = add_acc(v, shfl_x(v, o));
-  }
-  __syncthreads();
-  return v;  // valid in thread 0
-}
-
-// accumulator initialised from a stored element
-__device__ __forceinline__ double acc_of(double x) { return x; }
-__device__ __forceinline__ float2 acc_of(float2 x) { return x; }
-__device__ __forceinline__ float2 acc_of(float x) { return make_float2(x, 0.f); }
-
-__device__ __forceinline__ void amac(double& a, const double* cd, const float2*, int k, double x) {
-  a = fma(cd[k], x, a);
-}
-__device__ __forceinline__ void amac(float2& a, const double*, const float2* cf, int k, float2 x) {
-  df_mac(a, cf[k], x);
-}
-__device__ __forceinline__ void amac(float2& a, const double*, const float2* cf, int k, float x) {
-  df_mac1(a, cf[k], x);
-}
-
-__device__ __forceinline__ double store_v(double a, double*) { return a; }
-__device__ __forceinline__ float2 store_v(float2 a, float2*) { return df_norm(a); }
-__device__ __forceinline__ float store_v(float2 a, float*) { return __fadd_rn(a.x, a.y); }
-
-template <class V>
-struct AccOf;
-template <>
-struct AccOf<double> { using T = double; };
-template <>
-struct AccOf<float2> { using T = float2; };
-template <>
-struct AccOf<float> { using T = float2; };
 
 // ------------------------------------------------ reductions
 // partial[b] = sum over this block's elements of x*y (as double)
@@ -94,89 +34,14 @@ __global__ void __launch_bounds__(kRedThreads) k_dot(const V* __restrict__ x, co
   if (threadIdx.x == 0) partial[blockIdx.x] = to_d(acc);
 }
 
-// Multi-dot of the chunk k0 .. k0 + KB - 1: partial[q * nb + b] = block b's
-// share of <V_{k0+q}, w>.
-template <class V, int KB>
-__global__ void __launch_bounds__(kRedThreads) k_multidot(const V* __restrict__ Vb, uint64_t stride, int k0,
-                                                          int nvec, const V* __restrict__ w, uint64_t n,
-                                                          double* __restrict__ partial) {
-  using A = typename AccOf<V>::T;
-  __shared__ A sh[32];
-  A acc[KB];
-#pragma unroll
-  for (int q = 0; q < KB; ++q) acc[q] = A{};
-  int kn = min(KB, nvec - k0);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    V wi = w[i];
-#pragma unroll
-    for (int q = 0; q < KB; ++q)
-      if (q < kn) dmac(acc[q], Vb[(uint64_t)(k0 + q) * stride + i], wi);
-  }
-  for (int q = 0; q < kn; ++q) {
-    A r = block_reduce(acc[q], sh);
-    if (threadIdx.x == 0) partial[(uint64_t)q * gridDim.x + blockIdx.x] = to_d(r);
-  }
-}
-
-// The same multi-dot with sixteen-byte loads (every slot, and w, 16-byte
-// aligned): (KB + 1) x 16 bytes per thread in flight; the tail of the range
-// element by element.
-template <class V, int KB>
-__global__ void __launch_bounds__(kRedThreads) k_multidot16(const V* __restrict__ Vb, uint64_t stride, int k0,
-                                                            int nvec, const V* __restrict__ w, uint64_t n,
-                                                            double* __restrict__ partial) {
-  using A = typename AccOf<V>::T;
-  using W16 = Vec16<V>;
-  using VT = typename W16::T;
-  constexpr int N = W16::N;
-  __shared__ A sh[32];
-  A acc[KB];
-#pragma unroll
-  for (int q = 0; q < KB; ++q) acc[q] = A{};
-  const int kn = min(KB, nvec - k0);
-  const uint64_t nv = n / N;
-  const uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (uint64_t)gridDim.x * blockDim.x;
-  const VT* wv = reinterpret_cast<const VT*>(w);
-  const V* vk = Vb + (uint64_t)k0 * stride;
-  for (uint64_t t = g0; t < nv; t += gs) {
-    const VT wq = wv[t];
-    VT vq[KB];
-#pragma unroll
-    for (int q = 0; q < KB; ++q)
-      if (q < kn) vq[q] = __ldg(reinterpret_cast<const VT*>(vk + (uint64_t)q * stride) + t);
-#pragma unroll
-    for (int q = 0; q < KB; ++q)
-      if (q < kn) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) dmac(acc[q], W16::get(vq[q], i), W16::get(wq, i));
-      }
-  }
-  for (uint64_t i = nv * N + g0; i < n; i += gs) {
-    const V wi = w[i];
-#pragma unroll
-    for (int q = 0; q < KB; ++q)
-      if (q < kn) dmac(acc[q], vk[(uint64_t)q * stride + i], wi);
-  }
-  for (int q = 0; q < kn; ++q) {
-    A r = block_reduce(acc[q], sh);
-    if (threadIdx.x == 0) partial[(uint64_t)q * gridDim.x + blockIdx.x] = to_d(r);
-  }
-}
-
 // ------------------------------------------------ coefficient bookkeeping
 struct Coefs {
   double* alpha;    // [m+1]
   double* beta;     // [m+2], beta[0] = 0
-  double* nal_d;    // -alpha
-  float2* nal_f;
-  double* nbe_d;    // -beta
-  float2* nbe_f;
   double* inv_d;    // 1 / beta (0 when beta vanished)
   float2* inv_f;
   double* h_d;      // -h (CGS projections)
-  float2* h_f;
-  double* scale;    // running max |alpha|, beta
+  double* scale;    // running max |alpha|, beta (two slots: k_scale_beta reads one and writes the other)
   int* exhausted;   // first step with a vanished beta, -1 if none
   double* out;      // generic scalar output slots
   // three-vector recurrence on unnormalised vectors q_j (v_j = sigma_j q_j):
@@ -191,8 +56,7 @@ struct Coefs {
   int* step;        // device step index for graph-replayed steps (slot < 0 / j < 0 read it)
 };
 
-enum FinishOp { OP_SUM = 0, OP_ALPHA = 1, OP_BETA = 2, OP_NEGH = 3, OP_NORM_INV = 4, OP_SIGMA0 = 5,
-                OP_ALPHA_Q = 6, OP_BETA_Q = 7 };
+enum FinishOp { OP_SUM, OP_NEGH, OP_NORM_INV, OP_SIGMA0, OP_ALPHA_Q, OP_BETA_Q };
 
 // Sum nb partials (one output per block of this kernel) and apply `op`.
 __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict__ partial, int nb, int op,
@@ -206,29 +70,8 @@ __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict
   if (slot < 0) slot = *c.step + (-slot - 1);  // -1: current step j, -2: j + 1
   switch (op) {
     case OP_SUM: c.out[slot + o] = v; break;
-    case OP_ALPHA:
-      c.alpha[slot] = v;
-      c.nal_d[slot] = -v;
-      c.nal_f[slot] = df_from_double(-v);
-      *c.scale = fmax(*c.scale, fabs(v));
-      break;
-    case OP_BETA: {
-      double b = sqrt(fmax(v, 0.0));
-      double sc = fmax(*c.scale, b);
-      *c.scale = sc;
-      bool dead = !(b > thr * fmax(sc, 1.0));
-      if (dead && *c.exhausted < 0) *c.exhausted = slot;
-      c.beta[slot] = dead ? 0.0 : b;
-      c.nbe_d[slot] = dead ? 0.0 : -b;
-      c.nbe_f[slot] = df_from_double(dead ? 0.0 : -b);
-      double inv = dead ? 0.0 : 1.0 / b;
-      c.inv_d[slot] = inv;
-      c.inv_f[slot] = df_from_double(inv);
-      break;
-    }
     case OP_NEGH:
       c.h_d[slot + o] = -v;
-      c.h_f[slot + o] = df_from_double(-v);
       break;
     case OP_NORM_INV: {
       double b = sqrt(fmax(v, 0.0));
@@ -274,19 +117,6 @@ __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict
 }
 
 // ------------------------------------------------ vector updates
-// w = w - alpha_j v - beta_j vprev  (coefficients read from device memory)
-template <class V>
-__global__ void k_lz_update(V* __restrict__ w, const V* __restrict__ v, const V* __restrict__ vp, uint64_t n,
-                            Coefs c, int j) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    auto a = acc_of(w[i]);
-    amac(a, c.nal_d, c.nal_f, j, v[i]);
-    if (vp) amac(a, c.nbe_d, c.nbe_f, j, vp[i]);
-    w[i] = store_v(a, w);
-  }
-}
-
 // q_out = ua_j y + ub_j q_j + uc_j q_{j-1} with block partials of |q_out|^2.
 // q_out may be the buffer of q_{j-1} (element-wise in place).
 template <class V>
@@ -325,53 +155,6 @@ __global__ void k_scale_ritz(const double* __restrict__ S, const double* __restr
   Sqf[(size_t)i * ldS + j] = df_from_double(v);
 }
 
-// w -= sum_k h_k V_k for k in [0, nvec)
-template <class V>
-__global__ void k_multi_axpy(const V* __restrict__ Vb, uint64_t stride, int nvec, V* __restrict__ w, uint64_t n,
-                             Coefs c) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    auto a = acc_of(w[i]);
-    for (int k = 0; k < nvec; ++k) amac(a, c.h_d, c.h_f, k, Vb[(uint64_t)k * stride + i]);
-    w[i] = store_v(a, w);
-  }
-}
-
-// The same update with sixteen-byte loads and stores (slots and w 16-byte
-// aligned); each element's terms in the order k = 0 .. nvec - 1, as above.
-template <class V>
-__global__ void k_multi_axpy16(const V* __restrict__ Vb, uint64_t stride, int nvec, V* __restrict__ w, uint64_t n,
-                               Coefs c) {
-  using A = typename AccOf<V>::T;
-  using W16 = Vec16<V>;
-  using VT = typename W16::T;
-  constexpr int N = W16::N;
-  const uint64_t nv = n / N;
-  const uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (uint64_t)gridDim.x * blockDim.x;
-  VT* wv = reinterpret_cast<VT*>(w);
-  for (uint64_t t = g0; t < nv; t += gs) {
-    const VT wq = wv[t];
-    A a[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = acc_of(W16::get(wq, i));
-#pragma unroll 4
-    for (int k = 0; k < nvec; ++k) {
-      const VT vq = __ldg(reinterpret_cast<const VT*>(Vb + (uint64_t)k * stride) + t);
-#pragma unroll
-      for (int i = 0; i < N; ++i) amac(a[i], c.h_d, c.h_f, k, W16::get(vq, i));
-    }
-    VT o;
-#pragma unroll
-    for (int i = 0; i < N; ++i) W16::set(o, i, store_v(a[i], w));
-    wv[t] = o;
-  }
-  for (uint64_t i = nv * N + g0; i < n; i += gs) {
-    auto a = acc_of(w[i]);
-    for (int k = 0; k < nvec; ++k) amac(a, c.h_d, c.h_f, k, Vb[(uint64_t)k * stride + i]);
-    w[i] = store_v(a, w);
-  }
-}
-
 // out = w * inv[slot]
 template <class V>
 __global__ void k_scale(const V* __restrict__ w, V* __restrict__ out, uint64_t n, Coefs c, int slot) {
@@ -380,6 +163,52 @@ __global__ void k_scale(const V* __restrict__ w, V* __restrict__ out, uint64_t n
     typename AccOf<V>::T a{};
     amac(a, c.inv_d, c.inv_f, slot, w[i]);
     out[i] = store_v(a, out);
+  }
+}
+
+// beta_{j+1} = |w| from its nb partials, and out = w / beta_{j+1} (zeros where
+// beta vanished).  Every block sums the partials itself, in the same order, so
+// that the step needs no launch for one number; block 0 keeps beta_{j+1}, the
+// running scale (slot 1 - ph; every block reads slot ph) and the first
+// vanished step.
+template <class V>
+__global__ void __launch_bounds__(kRedThreads) k_scale_beta(const V* __restrict__ w, V* __restrict__ out, uint64_t n,
+                                                            const double* __restrict__ partial, int nb, Coefs c,
+                                                            int slot, int ph, double thr) {
+  using A = typename AccOf<V>::T;
+  using W16 = Vec16<V>;
+  using VT = typename W16::T;
+  __shared__ double sh[32];
+  const double b = sqrt(fmax(block_total(partial, nb, sh), 0.0));
+  const double sc = fmax(c.scale[ph], b);
+  const bool dead = !(b > thr * fmax(sc, 1.0));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    c.scale[1 - ph] = sc;
+    if (dead && *c.exhausted < 0) *c.exhausted = slot;
+    c.beta[slot] = dead ? 0.0 : b;
+  }
+  A inv;
+  h_split(inv, dead ? 0.0 : 1.0 / b);
+  const uint64_t nv = (n + W16::N - 1) / W16::N;
+  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t e0 = t * W16::N;
+    if (e0 + W16::N <= n) {
+      const VT q = reinterpret_cast<const VT*>(w)[t];
+      VT o{};
+#pragma unroll
+      for (int i = 0; i < W16::N; ++i) {
+        A a{};
+        hmac(a, inv, W16::get(q, i));
+        W16::set(o, i, store_v(a, out));
+      }
+      reinterpret_cast<VT*>(out)[t] = o;
+    } else {
+      for (uint64_t e = e0; e < n; ++e) {
+        A a{};
+        hmac(a, inv, w[e]);
+        out[e] = store_v(a, out);
+      }
+    }
   }
 }
 
@@ -479,6 +308,8 @@ struct Work {
   uint32_t grid;
   double* partial;  // ctx->d_red
   Coefs c;
+  double* hpart = nullptr;  // projections' partials (reorthogonalised solvers)
+  int ph = 0;               // which slot of c.scale is current
 };
 
 template <class V>
@@ -489,27 +320,88 @@ int dot_to(Work<V>& W, const V* x, const V* y, int op, int slot, double thr = 0.
   return ED_OK;
 }
 
-// CGS2 against basis vectors [0, nvec): twice h = V^T w, w -= V h.  The
-// projections are reduced eight at a time, so every chunk runs on the full
-// grid whatever the basis size.
+// Full reorthogonalisation of w against the basis vectors [0, nvec), every slot
+// and w starting on a 16-byte boundary: twice h = V^T w, w -= V h, with the
+// three-term update of lz (if any) ahead of the first projection; W.partial
+// gets the cgs_grid() partials of the final <w, w>.  Three sweeps over the
+// basis instead of four: the first update and the second projection share
+// one, in which a tile's second read comes from L2.
 template <class V>
-int cgs2(Work<V>& W, const V* Vb, uint64_t stride, int nvec, V* w) {
-  if (nvec <= 0) return ED_OK;
-  constexpr int KB = 8;
-  const int nb = (int)std::min<uint64_t>(W.grid, (uint64_t)kRedSlots / KB);
-  // sixteen-byte loads when every slot and w start on a 16-byte boundary
-  const bool v16 = (stride * sizeof(V)) % 16 == 0 && reinterpret_cast<uintptr_t>(Vb) % 16 == 0 &&
-                   reinterpret_cast<uintptr_t>(w) % 16 == 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int k0 = 0; k0 < nvec; k0 += KB) {
-      if (v16) k_multidot16<V, KB><<<nb, kRedThreads, 0, W.st>>>(Vb, stride, k0, nvec, w, W.n, W.partial);
-      else k_multidot<V, KB><<<nb, kRedThreads, 0, W.st>>>(Vb, stride, k0, nvec, w, W.n, W.partial);
-      k_finish<<<std::min(KB, nvec - k0), kRedThreads, 0, W.st>>>(W.partial, nb, OP_NEGH, k0, W.c, 0.0);
+int cgs2(Work<V>& W, const V* Vb, uint64_t stride, int nvec, V* w, LzTerm<V> lz = LzTerm<V>()) {
+  const uint32_t nb = cgs_grid<V>(W.ctx, W.n);
+  const LzTerm<V> none;
+  auto finish = [&](int k0, int kn) {
+    k_finish<<<kn, kRedThreads, 0, W.st>>>(W.hpart, (int)nb, OP_NEGH, k0, W.c, 0.0);
+  };
+  auto dots = [&](int k0, int kn, int rev, const LzTerm<V>& t) {
+    k_cgs<V, false, true><<<nb, kCgsThreads, cgs_smem<V>(kn, false, true), W.st>>>(
+        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, nullptr, W.hpart, nullptr, t);
+    finish(k0, kn);
+  };
+  auto update = [&](int k0, int kn, int rev) {
+    k_cgs<V, true, false><<<nb, kCgsThreads, cgs_smem<V>(kn, true, false), W.st>>>(
+        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, W.c.h_d + k0, nullptr, W.partial, none);
+  };
+  if (nvec <= kCgsMaxVec) {
+    dots(0, nvec, 0, lz);
+    k_cgs<V, true, true><<<nb, kCgsThreads, cgs_smem<V>(nvec, true, true), W.st>>>(
+        Vb, stride, nvec, w, W.n, 1, W.c.h_d, W.hpart, nullptr, none);
+    finish(0, nvec);
+    update(0, nvec, 0);
+  } else {   // a basis of more vectors than a block's shared memory serves at once: range by range
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int k0 = 0; k0 < nvec; k0 += kCgsMaxVec)
+        dots(k0, std::min(kCgsMaxVec, nvec - k0), 0, pass == 0 && k0 == 0 ? lz : none);
+      for (int k0 = 0; k0 < nvec; k0 += kCgsMaxVec) update(k0, std::min(kCgsMaxVec, nvec - k0), 0);
     }
-    if (v16) k_multi_axpy16<V><<<W.grid, 256, 0, W.st>>>(Vb, stride, nvec, w, W.n, W.c);
-    else k_multi_axpy<V><<<W.grid, 256, 0, W.st>>>(Vb, stride, nvec, w, W.n, W.c);
-    ED_LAUNCH_CHECK();
   }
+  ED_LAUNCH_CHECK();
+  return ED_OK;
+}
+
+// Doubles of Work::hpart for a basis of mmax + 1 vectors.
+template <class V>
+size_t cgs_part(const Ctx* c, uint64_t n, int mmax) {
+  return (size_t)std::min(mmax + 1, kCgsMaxVec) * cgs_grid<V>(c, n);
+}
+
+// H v_j with the partials of <v_j, H v_j> in W.partial; *np of them.
+template <class V>
+int apply_dot(const Sector* s, Work<V>& W, const V* x, V* y, int* np) {
+  if (s->fast.ok) return apply_fast(s, x, y, W.st, W.partial, np);
+  ED_TRY(apply_h(s, x, y, W.st));
+  k_dot<V><<<W.grid, kRedThreads, 0, W.st>>>(x, y, W.n, W.partial);
+  ED_LAUNCH_CHECK();
+  *np = (int)W.grid;
+  return ED_OK;
+}
+
+// One reorthogonalised Lanczos step: w = H v, the three-term update (with vp
+// unless NULL), CGS2 against [0, j], beta_{j+1} and v_{j+1} = w / beta_{j+1}.
+// e0, e1 bracket the H*v.
+template <class V>
+int lanczos_step(const Sector* s, Work<V>& W, const V* Vb, uint64_t ld, int j, const V* vp, V* w, V* vnext, double thr,
+                 cudaEvent_t e0, cudaEvent_t e1) {
+  const V* vj = Vb + (uint64_t)j * ld;
+  int np = 0;
+  ED_TRY_CUDA(cudaEventRecord(e0, W.st));
+  ED_TRY(apply_dot(s, W, vj, w, &np));
+  ED_TRY_CUDA(cudaEventRecord(e1, W.st));
+  LzTerm<V> lz;
+  lz.v = vj;
+  lz.vp = vp;
+  lz.apart = W.partial;
+  lz.na = np;
+  lz.alpha = W.c.alpha + j;
+  lz.beta = W.c.beta + j;
+  lz.scale = W.c.scale + W.ph;
+  ED_TRY(cgs2(W, Vb, ld, j + 1, w, lz));
+  const uint32_t grid =
+      (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((W.n / Vec16<V>::N + 255) / 256, (uint64_t)W.ctx->num_sms * 8));
+  k_scale_beta<V><<<grid, kRedThreads, 0, W.st>>>(w, vnext, W.n, W.partial, (int)cgs_grid<V>(W.ctx, W.n), W.c, j + 1,
+                                                 W.ph, thr);
+  ED_LAUNCH_CHECK();
+  W.ph ^= 1;
   return ED_OK;
 }
 
@@ -550,15 +442,10 @@ Coefs carve_coefs(Carve& cv, int mmax) {
   size_t m2 = (size_t)mmax + 2;
   c.alpha = cv.take<double>(m2);
   c.beta = cv.take<double>(m2);
-  c.nal_d = cv.take<double>(m2);
-  c.nal_f = cv.take<float2>(m2);
-  c.nbe_d = cv.take<double>(m2);
-  c.nbe_f = cv.take<float2>(m2);
   c.inv_d = cv.take<double>(m2);
   c.inv_f = cv.take<float2>(m2);
   c.h_d = cv.take<double>(m2);
-  c.h_f = cv.take<float2>(m2);
-  c.scale = cv.take<double>(1);
+  c.scale = cv.take<double>(2);
   c.exhausted = cv.take<int>(1);
   c.out = cv.take<double>(64);
   c.sigma = cv.take<double>(m2);
@@ -576,20 +463,15 @@ __global__ void k_init_coefs(Coefs c, int m2) {
   for (int i = threadIdx.x; i < m2; i += blockDim.x) {
     c.alpha[i] = 0;
     c.beta[i] = 0;
-    c.nal_d[i] = 0;
-    c.nal_f[i] = make_float2(0, 0);
-    c.nbe_d[i] = 0;
-    c.nbe_f[i] = make_float2(0, 0);
     c.inv_d[i] = 0;
     c.inv_f[i] = make_float2(0, 0);
     c.h_d[i] = 0;
-    c.h_f[i] = make_float2(0, 0);
     c.sigma[i] = 0;
     c.ua_d[i] = c.ub_d[i] = c.uc_d[i] = 0;
     c.ua_f[i] = c.ub_f[i] = c.uc_f[i] = make_float2(0, 0);
   }
   if (threadIdx.x == 0) {
-    *c.scale = 0.0;
+    c.scale[0] = c.scale[1] = 0.0;
     *c.exhausted = -1;
     *c.step = 0;
   }
@@ -613,23 +495,22 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   Ctx* ctx = s->ctx;
   const uint64_t n = s->dim;
   const int k = o->k;
-  const int reorth = o->reorth ? 1 : 0;
   int mmax = (int)std::min<uint64_t>((uint64_t)o->max_iter, n);
   if (mmax < 1) mmax = 1;
   const int check_every = std::max(1, o->check_every);
   const int kk = std::min<int>(k, (int)n);
 
-  // workspace: basis (mmax + 1 vectors with reorthogonalisation, else 3), w
+  // workspace: basis of mmax + 1 vectors, w
   size_t eb = sizeof(V);
-  int nvec_store = reorth ? (mmax + 1) : 3;
-  DevBuf vb, cb, v0b;
+  const int nvec_store = mmax + 1;
+  DevBuf vb, cb, hb;
   // basis slots padded to 32 elements, so that each starts 16-byte aligned
   const uint64_t ld = pad32(n);
   ED_TRY(vb.alloc(ctx, ((size_t)nvec_store + 1) * ld * eb));
   ED_TRY(cb.alloc(ctx, coef_bytes(mmax, std::max(kk, 1))));
   V* Vbase = static_cast<V*>(vb.p);
   V* w = Vbase + (size_t)nvec_store * ld;
-  if (!reorth) ED_TRY(v0b.alloc(ctx, n * eb));
+  ED_TRY(hb.alloc(ctx, cgs_part<V>(ctx, n, mmax) * sizeof(double)));
   Carve cv{static_cast<char*>(cb.p)};
   Coefs c = carve_coefs(cv, mmax);
   int ldS = mmax + 1;
@@ -647,11 +528,12 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   if (W.grid == 0) W.grid = 1;
   W.partial = ctx->d_red;
   W.c = c;
+  W.hpart = static_cast<double*>(hb.p);
   uint32_t vgrid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 16);
   if (vgrid == 0) vgrid = 1;
 
   k_init_coefs<<<1, 256, 0, st>>>(c, mmax + 2);
-  auto vec = [&](int j) -> V* { return reorth ? Vbase + (size_t)j * ld : Vbase + (size_t)(j % 3) * ld; };
+  auto vec = [&](int j) -> V* { return Vbase + (size_t)j * ld; };
 
   // start vector
   if (o->v0) {
@@ -662,7 +544,6 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   ED_TRY(dot_to(W, (const V*)w, (const V*)w, OP_NORM_INV, 0));
   k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(0), n, c, 0);
   ED_LAUNCH_CHECK();
-  if (!reorth) ED_TRY_CUDA(cudaMemcpyAsync(v0b.p, vec(0), n * eb, cudaMemcpyDeviceToDevice, st));
 
   // one event pair per step to time the H*v launches
   std::vector<cudaEvent_t> evs(2 * (size_t)mmax);
@@ -689,19 +570,9 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   while (!done) {
     exhausted = false;
     for (; j < mmax; ++j) {
-      V* vj = vec(j);
-      V* vjm = (j > 0) ? vec(j - 1) : nullptr;
-      ED_TRY_CUDA(cudaEventRecord(evs[2 * j], st));
-      ED_TRY(apply_h(s, vj, w, st));
-      ED_TRY_CUDA(cudaEventRecord(evs[2 * j + 1], st));
+      ED_TRY(lanczos_step(s, W, (const V*)Vbase, ld, j, j > 0 ? vec(j - 1) : nullptr, w, vec(j + 1), thr, evs[2 * j],
+                          evs[2 * j + 1]));
       n_timed = std::max(n_timed, j + 1);
-      ED_TRY(dot_to(W, (const V*)vj, (const V*)w, OP_ALPHA, j));
-      k_lz_update<V><<<vgrid, 256, 0, st>>>(w, vj, vjm, n, c, j);
-      ED_LAUNCH_CHECK();
-      if (reorth) ED_TRY(cgs2(W, (const V*)Vbase, ld, j + 1, w));
-      ED_TRY(dot_to(W, (const V*)w, (const V*)w, OP_BETA, j + 1, thr));
-      k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(j + 1), n, c, j + 1);
-      ED_LAUNCH_CHECK();
       m = j + 1;
       bool check = ((m % check_every) == 0) || (m == mmax) || (n <= 4096);
       if (!check) continue;
@@ -757,7 +628,7 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
       for (int i = 0; i < kc; ++i) h_res[i] = 0.0;
       n_conv = kc;
       beta_last = 0.0;
-      if (!reorth || (uint64_t)m >= n || m >= mmax || kc >= kk) {
+      if ((uint64_t)m >= n || m >= mmax || kc >= kk) {
         done = true;
         break;
       }
@@ -765,15 +636,12 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
       ++restarts;
       k_random<V><<<vgrid, 256, 0, st>>>(w, n, o->seed + 7919ull * restarts);
       ED_TRY(cgs2(W, (const V*)Vbase, ld, m, w));
-      ED_TRY(dot_to(W, (const V*)w, (const V*)w, OP_NORM_INV, 1));
+      k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c, 0.0);
       k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(m), n, c, 1);
       // beta[m] = 0 splits T; reset the exhaustion flag
       double zero = 0.0;
       int neg = -1;
       ED_TRY_CUDA(cudaMemcpyAsync(c.beta + m, &zero, sizeof(double), cudaMemcpyHostToDevice, st));
-      ED_TRY_CUDA(cudaMemcpyAsync(c.nbe_d + m, &zero, sizeof(double), cudaMemcpyHostToDevice, st));
-      float2 zf = make_float2(0.f, 0.f);
-      ED_TRY_CUDA(cudaMemcpyAsync(c.nbe_f + m, &zf, sizeof(float2), cudaMemcpyHostToDevice, st));
       ED_TRY_CUDA(cudaMemcpyAsync(c.exhausted, &neg, sizeof(int), cudaMemcpyHostToDevice, st));
       ED_TRY_CUDA(cudaStreamSynchronize(st));
       j = m;
@@ -792,25 +660,9 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
     // S for the final m
     ED_TRY(tridiag(ctx, st, c, m, kc, 0.0, theta, Sd, Sf, ldS, resid, twork));
     V* out = static_cast<V*>(evecs);
-    if (reorth) {
-      for (int i0 = 0; i0 < kc; i0 += 8)
-        k_ritz<V, 8><<<vgrid, 256, 0, st>>>(Vbase, ld, m, Sd, Sf, ldS, i0, std::min(8, kc - i0), out, n, 0);
-      ED_LAUNCH_CHECK();
-    } else {
-      // second pass: regenerate v_j with the stored alpha, beta and accumulate
-      ED_TRY_CUDA(cudaMemsetAsync(out, 0, (size_t)kc * n * eb, st));
-      ED_TRY_CUDA(cudaMemcpyAsync(vec(0), v0b.p, n * eb, cudaMemcpyDeviceToDevice, st));
-      for (int jj = 0; jj < m; ++jj) {
-        for (int i0 = 0; i0 < kc; i0 += 8)
-          k_ritz<V, 8><<<vgrid, 256, 0, st>>>(vec(jj), n, 1, Sd + jj, Sf + jj, ldS, i0, std::min(8, kc - i0), out,
-                                              n, 1);
-        if (jj + 1 == m) break;
-        ED_TRY(apply_h(s, vec(jj), w, st));
-        k_lz_update<V><<<vgrid, 256, 0, st>>>(w, vec(jj), jj > 0 ? vec(jj - 1) : nullptr, n, c, jj);
-        k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(jj + 1), n, c, jj + 1);
-        ED_LAUNCH_CHECK();
-      }
-    }
+    for (int i0 = 0; i0 < kc; i0 += 8)
+      k_ritz<V, 8><<<vgrid, 256, 0, st>>>(Vbase, ld, m, Sd, Sf, ldS, i0, std::min(8, kc - i0), out, n, 0);
+    ED_LAUNCH_CHECK();
   }
   ED_TRY_CUDA(cudaStreamSynchronize(st));
   for (int q = 0; q < n_timed; ++q) {

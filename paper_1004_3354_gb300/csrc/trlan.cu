@@ -194,11 +194,12 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
 
   // basis V[0..m] (m + 1 vectors), w, rotation target T[0..keep)
   const int n_rot = (m >= 3) ? keep : 0;
-  DevBuf vb, cb;
+  DevBuf vb, cb, hb;
   // slots padded to 32 elements, so that each starts 16-byte aligned
   const uint64_t ld = pad32(n);
   ED_TRY(vb.alloc(ctx, ((size_t)m + 2 + n_rot) * ld * eb));
   ED_TRY(cb.alloc(ctx, coef_bytes(m, 1) + (size_t)kMaxBasis * kMaxBasis * 8 * 4 + (size_t)kMaxBasis * 8 * 8));
+  ED_TRY(hb.alloc(ctx, cgs_part<V>(ctx, n, m) * sizeof(double)));
   V* Vb = static_cast<V*>(vb.p);
   V* w = Vb + (size_t)(m + 1) * ld;
   V* T = w + ld;  // rotation target, keep vectors of n elements back to back
@@ -221,6 +222,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   if (W.grid == 0) W.grid = 1;
   W.partial = ctx->d_red;
   W.c = c;
+  W.hpart = static_cast<double*>(hb.p);
   uint32_t vgrid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 16);
   if (vgrid == 0) vgrid = 1;
   auto vec = [&](int j) -> V* { return Vb + (size_t)j * ld; };
@@ -262,17 +264,9 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   int j = 0;  // next basis slot to extend from
   while (!done) {
     while (j < m) {
-      ED_TRY_CUDA(cudaEventRecord(evs[2 * j], st));
-      ED_TRY(apply_h(s, vec(j), w, st));
-      ED_TRY_CUDA(cudaEventRecord(evs[2 * j + 1], st));
+      ED_TRY(lanczos_step(s, W, (const V*)Vb, ld, j, j > l ? vec(j - 1) : nullptr, w, vec(j + 1), thr, evs[2 * j],
+                          evs[2 * j + 1]));
       pending.push_back(j);
-      ED_TRY(dot_to(W, (const V*)vec(j), (const V*)w, OP_ALPHA, j));
-      k_lz_update<V><<<vgrid, 256, 0, st>>>(w, vec(j), j > l ? vec(j - 1) : nullptr, n, c, j);
-      ED_LAUNCH_CHECK();
-      ED_TRY(cgs2(W, (const V*)Vb, ld, j + 1, w));
-      ED_TRY(dot_to(W, (const V*)w, (const V*)w, OP_BETA, j + 1, thr));
-      k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(j + 1), n, c, j + 1);
-      ED_LAUNCH_CHECK();
       ++iters;
       size = ++j;
       if (size < m && ((size - l) % check_every) != 0 && iters < max_iter) continue;
@@ -312,15 +306,12 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
         ++injections;
         k_random<V><<<vgrid, 256, 0, st>>>(w, n, o->seed + 7919ull * (uint64_t)injections);
         ED_TRY(cgs2(W, (const V*)Vb, ld, size, w));
-        ED_TRY(dot_to(W, (const V*)w, (const V*)w, OP_NORM_INV, 1));
+        k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c, 0.0);
         k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(size), n, c, 1);
         ED_LAUNCH_CHECK();
         const double zero = 0.0;
-        const float2 zf = make_float2(0.f, 0.f);
         const int neg = -1;
         ED_TRY_CUDA(cudaMemcpyAsync(c.beta + size, &zero, sizeof(double), cudaMemcpyHostToDevice, st));
-        ED_TRY_CUDA(cudaMemcpyAsync(c.nbe_d + size, &zero, sizeof(double), cudaMemcpyHostToDevice, st));
-        ED_TRY_CUDA(cudaMemcpyAsync(c.nbe_f + size, &zf, sizeof(float2), cudaMemcpyHostToDevice, st));
         ED_TRY_CUDA(cudaMemcpyAsync(c.exhausted, &neg, sizeof(int), cudaMemcpyHostToDevice, st));
         ED_TRY_CUDA(cudaStreamSynchronize(st));
         continue;  // j == size: the next step starts from the new vector (a full basis restarts first)
