@@ -433,29 +433,26 @@ __global__ void k_b_ritz(BatchDev B, const V* __restrict__ Vb, const double* __r
 }
 
 // --------------------------------------------------- batched tridiagonal solve
-__global__ void k_bt_eig(const double* __restrict__ alpha, const double* __restrict__ beta, int ms,
-                         const int* __restrict__ mj, const int* __restrict__ kj, int kmax, double* __restrict__ theta) {
+__global__ void __launch_bounds__(32) k_bt_pair(const double* __restrict__ alpha, const double* __restrict__ beta,
+                                                int ms, const int* __restrict__ active,
+                                                const int* __restrict__ mj, const int* __restrict__ kj, int kmax,
+                                                double* __restrict__ theta, double* __restrict__ S,
+                                                double* __restrict__ work) {
+  extern __shared__ __align__(16) double trish[];
   const int i = blockIdx.x, job = blockIdx.y;
-  if (i >= kj[job] || i >= mj[job]) return;
-  tri_eig_one(alpha + (size_t)job * ms, beta + (size_t)job * ms, mj[job], i, theta + (size_t)job * kmax);
+  // a converged job keeps the pairs of the check at which it converged
+  if (!active[job] || i >= kj[job] || i >= mj[job]) return;
+  const size_t row = (size_t)job * kmax;
+  tri_pair_one(alpha + (size_t)job * ms, beta + (size_t)job * ms, mj[job], i, theta + row, S + row * ms, ms,
+               work + row * 6 * ms, trish);
 }
 
-__global__ void k_bt_vec(const double* __restrict__ alpha, const double* __restrict__ beta, int ms,
-                         const int* __restrict__ mj, const int* __restrict__ kj, int kmax, const double* __restrict__ theta,
-                         double* __restrict__ S, double* __restrict__ work) {
-  const int i = blockIdx.x, job = blockIdx.y;
-  if (threadIdx.x != 0 || i >= kj[job] || i >= mj[job]) return;
-  const int ldS = ms;
-  tri_vec_one(alpha + (size_t)job * ms, beta + (size_t)job * ms, mj[job], theta + (size_t)job * kmax,
-              S + (size_t)job * kmax * ldS, ldS, work + (size_t)job * kmax * 6 * ldS, i);
-}
-
-__global__ void k_bt_finish(const double* __restrict__ beta, int ms, const int* __restrict__ mj,
-                            const int* __restrict__ kj, int kmax, const double* __restrict__ theta,
+__global__ void k_bt_finish(const double* __restrict__ beta, int ms, const int* __restrict__ active,
+                            const int* __restrict__ mj, const int* __restrict__ kj, int kmax, const double* __restrict__ theta,
                             double* __restrict__ S, float2* __restrict__ Sf, double* __restrict__ resid) {
   const int job = blockIdx.x;
   const int m = mj[job], k = min(kj[job], mj[job]);
-  if (m < 1 || k < 1) return;
+  if (!active[job] || m < 1 || k < 1) return;
   const int ldS = ms;
   tri_finish_block(theta + (size_t)job * kmax, k, m, beta[(size_t)job * ms + m], S + (size_t)job * kmax * ldS, ldS,
                    Sf + (size_t)job * kmax * ldS, resid + (size_t)job * kmax);
@@ -660,9 +657,9 @@ int batch_run(Batch* bt, const ed_lanczos_opts* o, double* evals, int* iters, ed
       h_m[q] = (h_ex[q] >= 0) ? h_ex[q] : steps;
     }
     ED_TRY_CUDA(cudaMemcpyAsync(dm, h_m.data(), sizeof(int) * J, cudaMemcpyHostToDevice, st));
-    k_bt_eig<<<dim3(kmax, J), 32, 0, st>>>(B.alpha, B.beta, ms, dm, dk, kmax, theta);
-    k_bt_vec<<<dim3(kmax, J), 32, 0, st>>>(B.alpha, B.beta, ms, dm, dk, kmax, theta, S, work);
-    k_bt_finish<<<J, 128, 0, st>>>(B.beta, ms, dm, dk, kmax, theta, S, Sf, resid);
+    k_bt_pair<<<dim3(kmax, J), 32, tri_smem(steps), st>>>(B.alpha, B.beta, ms, B.active, dm, dk, kmax, theta, S,
+                                                                work);
+    k_bt_finish<<<J, 128, 0, st>>>(B.beta, ms, B.active, dm, dk, kmax, theta, S, Sf, resid);
     ED_LAUNCH_CHECK();
     ED_TRY_CUDA(cudaMemcpyAsync(h_theta.data(), theta, sizeof(double) * J * kmax, cudaMemcpyDeviceToHost, st));
     ED_TRY_CUDA(cudaMemcpyAsync(h_res.data(), resid, sizeof(double) * J * kmax, cudaMemcpyDeviceToHost, st));

@@ -281,17 +281,12 @@ __global__ void k_copy_f64(const void* __restrict__ a, void* __restrict__ b, uin
 }
 
 // ------------------------------------------------ tridiagonal eigensolver
-// Eigenvalue blockIdx.x (ascending) by 32-way multisection, one warp per value.
-__global__ void k_tri_eig(const double* __restrict__ a, const double* __restrict__ b, int m,
-                          double* __restrict__ theta) {
-  tri_eig_one(a, b, m, blockIdx.x, theta);
-}
-
-// Inverse iteration for eigenvector blockIdx.x (thread 0 of the block).
-__global__ void k_tri_vec(const double* __restrict__ a, const double* __restrict__ b, int m,
-                          const double* __restrict__ theta, double* __restrict__ S, int ldS,
-                          double* __restrict__ work) {
-  if (threadIdx.x == 0) tri_vec_one(a, b, m, theta, S, ldS, work, blockIdx.x);
+// Eigenpair blockIdx.x (ascending), one warp per pair.
+__global__ void __launch_bounds__(32) k_tri_pair(const double* __restrict__ a, const double* __restrict__ b, int m,
+                                                 double* __restrict__ theta, double* __restrict__ S, int ldS,
+                                                 double* __restrict__ work) {
+  extern __shared__ __align__(16) double trish[];
+  tri_pair_one(a, b, m, blockIdx.x, theta, S, ldS, work, trish);
 }
 
 __global__ void k_tri_finish(const double* __restrict__ theta, int k, int m, double beta_m, double* __restrict__ S,
@@ -480,8 +475,7 @@ __global__ void k_init_coefs(Coefs c, int m2) {
 // Solve the m x m tridiagonal problem for its k lowest pairs.
 int tridiag(Ctx* ctx, cudaStream_t st, const Coefs& c, int m, int k, double beta_m, double* theta,
             double* S, float2* Sf, int ldS, double* resid, double* work) {
-  k_tri_eig<<<k, 32, 0, st>>>(c.alpha, c.beta, m, theta);
-  k_tri_vec<<<k, 32, 0, st>>>(c.alpha, c.beta, m, theta, S, ldS, work);
+  k_tri_pair<<<k, 32, tri_smem(m), st>>>(c.alpha, c.beta, m, theta, S, ldS, work);
   k_tri_finish<<<1, 128, 0, st>>>(theta, k, m, beta_m, S, ldS, Sf, resid);
   ED_LAUNCH_CHECK();
   (void)ctx;

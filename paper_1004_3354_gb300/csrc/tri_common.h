@@ -1,13 +1,26 @@
 // Tridiagonal eigensolver used by the Lanczos drivers (internal header):
-// Sturm-sequence multisection for the k lowest eigenvalues (one warp per
-// value), inverse iteration with tridiagonal Gaussian elimination and partial
-// pivoting for the eigenvectors, then Gram-Schmidt among (nearly) equal
+// Sturm-sequence multisection for the k lowest eigenvalues, inverse iteration
+// with tridiagonal Gaussian elimination and partial pivoting for their
+// vectors, one warp per pair; then Gram-Schmidt among (nearly) equal
 // eigenvalues.  All in FP64.
+//
+// Bound by the latency and the rate of FP64 instructions along the matrix
+// (GB300 issues about 1.6 FP64 lanes per SM and clock: 20 cycles per warp
+// instruction), so the chains are kept short: the Sturm counts use the
+// determinant recurrence (3 FP64 instructions per row and no division), the
+// matrix and the factors sit in shared memory, the factor's reciprocals are
+// taken by all lanes at once, and a pair's value and vector share one launch.
 #pragma once
 
 #include "ed_internal.h"
 
 namespace ed {
+
+constexpr int kTriSmemRows = 1024;   // matrices up to this size run from shared memory (6 doubles per row)
+
+inline size_t tri_smem(int m) {
+  return (size_t)6 * (m < 1 ? 1 : m < kTriSmemRows ? m : kTriSmemRows) * sizeof(double);
+}
 
 // Block-wide sum, result valid in thread 0.
 __device__ inline double tri_block_sum(double v, double* sh) {
@@ -24,128 +37,213 @@ __device__ inline double tri_block_sum(double v, double* sh) {
   return v;
 }
 
-// Sturm count: number of eigenvalues of T (alpha[0..m), beta[1..m)) below x.
-__device__ inline int sturm(const double* __restrict__ a, const double* __restrict__ b, int m, double x,
-                     double pivmin) {
-  int cnt = 0;
-  double q = a[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < 0) ++cnt;
-  for (int i = 1; i < m; ++i) {
-    q = (a[i] - x) - b[i] * b[i] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) ++cnt;
+__device__ __forceinline__ int tri_exp(double v) { return __double2hiint(v) & 0x7ff00000; }
+
+// 2^(-e) for the binary exponent field e of a normal double
+__device__ __forceinline__ double tri_pow2_inv(int field) { return __hiloint2double(0x7fe00000 - field, 0); }
+
+// Sturm count: eigenvalues below x of the matrix with rows ab[i] = (a_i, b_i^2),
+// entries of magnitude at most about 1.  Determinants of the leading minors,
+// p_i = (a_i - x) p_{i-1} - b_i^2 p_{i-2}, whose sign changes count the
+// negative pivots; a pivot p_i / p_{i-1} below 2^-100 in magnitude counts as
+// -2^-100 (a change of a_i far below rounding).  Every eight rows p is brought
+// back to about 1 by an exact power of two, so that it cannot leave the range
+// of a double (a row shrinks it by at most 2^-100 and at most triples it).
+__device__ inline int sturm(const double2* __restrict__ ab, int m, double x) {
+  double p0 = 1.0, p1 = ab[0].x - x;
+  if (tri_exp(p1) + (100 << 20) < tri_exp(p0)) p1 = -0x1p-100;
+  int cnt = p1 < 0.0 ? 1 : 0;
+  auto row = [&](const double2 r) {
+    double p = fma(r.x - x, p1, -(r.y * p0));
+    if (tri_exp(p) + (100 << 20) < tri_exp(p1)) p = -p1 * 0x1p-100;
+    cnt += (unsigned)(__double2hiint(p) ^ __double2hiint(p1)) >> 31;
+    p0 = p1;
+    p1 = p;
+  };
+  int i = 1;
+  for (; i + 8 <= m; i += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) row(ab[i + q]);
+    const double sc = tri_pow2_inv(max(tri_exp(p0), tri_exp(p1)));
+    p0 *= sc;
+    p1 *= sc;
   }
+  for (; i < m; ++i) row(ab[i]);
   return cnt;
 }
 
-// Eigenvalue `blockIdx.x` (ascending) by 32-way multisection, one warp per value.
-__device__ inline void tri_eig_one(const double* __restrict__ a, const double* __restrict__ b, int m, int i,
-                                   double* __restrict__ theta) {
-  int lane = threadIdx.x;
-  double lo = a[0], hi = a[0], bmax = 0.0;
-  for (int r = 0; r < m; ++r) {
-    double off = (r > 0 ? fabs(b[r]) : 0.0) + (r + 1 < m ? fabs(b[r + 1]) : 0.0);
+__device__ __forceinline__ double tri_warp_min(double v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ double tri_warp_max(double v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// Eigenvalue i (ascending) by 32-way multisection of the Gershgorin interval,
+// one warp per value; ab is scratch for m rows.  The matrix is scaled by an
+// exact power of two to entries of magnitude at most 1.
+__device__ inline double tri_eig_one(const double* __restrict__ a, const double* __restrict__ b, int m, int i,
+                                     double2* ab) {
+  const int lane = threadIdx.x;
+  double lo = INFINITY, hi = -INFINITY;
+  for (int r = lane; r < m; r += 32) {
+    const double off = (r > 0 ? fabs(b[r]) : 0.0) + (r + 1 < m ? fabs(b[r + 1]) : 0.0);
     lo = fmin(lo, a[r] - off);
     hi = fmax(hi, a[r] + off);
-    if (r > 0) bmax = fmax(bmax, fabs(b[r]));
   }
-  double scale = fmax(fabs(lo), fabs(hi));
-  double pivmin = fmax(1e-300, 1e-290 * bmax * bmax);
-  lo -= 1e-14 * scale + 1e-300;
-  hi += 1e-14 * scale + 1e-300;
+  lo = tri_warp_min(lo);
+  hi = tri_warp_max(hi);
+  const double scale = fmax(fabs(lo), fabs(hi));
+  const int ex = tri_exp(scale);
+  // exact power-of-two scaling (none for a zero, tiny or huge matrix)
+  const double inv = (ex > (30 << 20) && ex < (2000 << 20)) ? tri_pow2_inv(ex) : 1.0;
+  for (int r = lane; r < m; r += 32) {
+    const double br = r > 0 ? b[r] * inv : 0.0;
+    ab[r] = make_double2(a[r] * inv, br * br);
+  }
+  __syncwarp();
+  const double sc = scale * inv;
+  lo = lo * inv - (1e-14 * sc + 1e-300);
+  hi = hi * inv + (1e-14 * sc + 1e-300);
   for (int it = 0; it < 64; ++it) {
-    if (hi - lo <= 4e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300) break;
-    double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-    int c = sturm(a, b, m, x, pivmin);
+    if (hi - lo <= 4e-16 * fmax(fabs(lo), fabs(hi)) + 0x1p-62 * sc) break;
+    const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
+    const int c = sturm(ab, m, x);
     // first lane whose point has more than i eigenvalues below it
-    unsigned above = __ballot_sync(0xffffffffu, c > i);
-    int f = above ? __ffs(above) - 1 : 32;
-    double nlo = (f == 0) ? lo : lo + (hi - lo) * (double)f / 33.0;
-    double nhi = (f == 32) ? hi : lo + (hi - lo) * (double)(f + 1) / 33.0;
+    const unsigned above = __ballot_sync(0xffffffffu, c > i);
+    const int f = above ? __ffs(above) - 1 : 32;
+    const double nlo = (f == 0) ? lo : lo + (hi - lo) * (double)f / 33.0;
+    const double nhi = (f == 32) ? hi : lo + (hi - lo) * (double)(f + 1) / 33.0;
     lo = nlo;
     hi = nhi;
   }
-  if (lane == 0) theta[i] = 0.5 * (lo + hi);
+  __syncwarp();
+  return 0.5 * (lo + hi) / inv;
 }
 
-// Inverse iteration for eigenvector blockIdx.x: solve (T - theta I) x = x_prev
-// by tridiagonal Gaussian elimination with partial pivoting (row interchanges
-// as in LAPACK's gttrf/gtts2), three sweeps.  work holds 6*ldS doubles per
-// eigenvector.  Output S[i*ldS + j], j < m, normalised, largest entry positive.
-__device__ inline void tri_vec_one(const double* __restrict__ a, const double* __restrict__ b, int m,
-                                   const double* __restrict__ theta, double* __restrict__ S, int ldS,
-                                   double* __restrict__ work, int k) {
-  double* x = work + (size_t)k * 6 * ldS;
-  double* dl = x + ldS;
-  double* d = dl + ldS;
-  double* du = d + ldS;
-  double* du2 = du + ldS;
-  double* piv = du2 + ldS;
-  double* s = S + (size_t)k * ldS;
-  const double th = theta[k];
+// Vector of eigenvalue k = theta by inverse iteration: solve (T - theta I) x =
+// x_prev by tridiagonal Gaussian elimination with partial pivoting (row
+// interchanges as in LAPACK's gttrf/gtts2), three sweeps, one warp: lane 0 runs
+// the recurrences, all lanes the rest.  wk holds 6 * m doubles of scratch.
+// Output s[j], j < m, normalised, largest entry positive.
+__device__ inline void tri_vec_one(const double* __restrict__ a, const double* __restrict__ b, int m, double th, int k,
+                                   double* wk, double* __restrict__ s) {
+  const int lane = threadIdx.x;
+  double* x = wk;
+  double* dl = x + m;
+  double* rd = dl + m;     // pivots, then their reciprocals
+  double* du = rd + m;
+  double* du2 = du + m;
+  double* piv = du2 + m;
   double anorm = 0.0;
-  for (int r = 0; r < m; ++r)
-    anorm = fmax(anorm, fabs(a[r]) + (r > 0 ? fabs(b[r]) : 0.0) + (r + 1 < m ? fabs(b[r + 1]) : 0.0));
+  for (int r = lane; r < m; r += 32) {
+    const double off = (r > 0 ? fabs(b[r]) : 0.0) + (r + 1 < m ? fabs(b[r + 1]) : 0.0);
+    anorm = fmax(anorm, fabs(a[r]) + off);
+    // the elimination reads the matrix from here
+    x[r] = a[r] - th;
+    dl[r] = r + 1 < m ? b[r + 1] : 0.0;
+  }
+  anorm = tri_warp_max(anorm);
   const double tiny = 2.2e-16 * fmax(anorm, 1e-300);
-  for (int r = 0; r < m; ++r) {
-    d[r] = a[r] - th;
-    du[r] = (r + 1 < m) ? b[r + 1] : 0.0;
-    dl[r] = (r + 1 < m) ? b[r + 1] : 0.0;  // subdiagonal (symmetric)
-    du2[r] = 0.0;
-    piv[r] = 0.0;
-  }
-  for (int r = 0; r + 1 < m; ++r) {
-    if (fabs(d[r]) >= fabs(dl[r])) {
-      double f = (d[r] != 0.0) ? dl[r] / d[r] : 0.0;
-      dl[r] = f;
-      d[r + 1] -= f * du[r];
-    } else {
-      double f = d[r] / dl[r];
-      d[r] = dl[r];
-      dl[r] = f;
-      double t = du[r];
-      du[r] = d[r + 1];
-      d[r + 1] = t - f * d[r + 1];
-      if (r + 2 < m) {
-        du2[r] = du[r + 1];
-        du[r + 1] = -f * du[r + 1];
-      }
-      piv[r] = 1.0;
-    }
-  }
-  for (int r = 0; r < m; ++r)
-    if (fabs(d[r]) < tiny) d[r] = (d[r] < 0 ? -tiny : tiny);
-  for (int r = 0; r < m; ++r) x[r] = 1.0 + 0.01 * (double)((r * 7919 + k * 104729) % 97) / 97.0;
-  for (int sweep = 0; sweep < 3; ++sweep) {
+  __syncwarp();
+  if (lane == 0) {
+    double d = x[0], u = dl[0];   // the current row's diagonal and superdiagonal
     for (int r = 0; r + 1 < m; ++r) {
-      if (piv[r] == 0.0) {
-        x[r + 1] -= dl[r] * x[r];
+      const double sub = dl[r], nd = x[r + 1], nu = dl[r + 1];
+      if (fabs(d) >= fabs(sub)) {
+        const double f = (d != 0.0) ? sub / d : 0.0;
+        rd[r] = d;
+        dl[r] = f;
+        du[r] = u;
+        du2[r] = 0.0;
+        piv[r] = 0.0;
+        d = nd - f * u;
+        u = nu;
       } else {
-        double t = x[r];
-        x[r] = x[r + 1];
-        x[r + 1] = t - dl[r] * x[r];
+        const double f = d / sub;
+        rd[r] = sub;
+        dl[r] = f;
+        du[r] = nd;
+        du2[r] = nu;
+        piv[r] = 1.0;
+        d = u - f * nd;
+        u = -f * nu;
       }
     }
-    x[m - 1] /= d[m - 1];
-    if (m > 1) x[m - 2] = (x[m - 2] - du[m - 2] * x[m - 1]) / d[m - 2];
-    for (int r = m - 3; r >= 0; --r) x[r] = (x[r] - du[r] * x[r + 1] - du2[r] * x[r + 2]) / d[r];
+    rd[m - 1] = d;
+    du[m - 1] = du2[m - 1] = piv[m - 1] = 0.0;
+  }
+  __syncwarp();
+  for (int r = lane; r < m; r += 32) {
+    double d = rd[r];
+    if (fabs(d) < tiny) d = (d < 0 ? -tiny : tiny);
+    rd[r] = 1.0 / d;
+    x[r] = 1.0 + 0.01 * (double)((r * 7919 + k * 104729) % 97) / 97.0;
+  }
+  __syncwarp();
+  for (int sweep = 0; sweep < 3; ++sweep) {
+    if (lane == 0) {
+      double t = x[0];
+#pragma unroll 4
+      for (int r = 0; r + 1 < m; ++r) {
+        const double xn = x[r + 1], f = dl[r];
+        const bool pv = piv[r] != 0.0;
+        const double keep = pv ? xn : t, go = pv ? t : xn;
+        x[r] = keep;
+        t = go - f * keep;
+      }
+      double x1 = t * rd[m - 1], x2 = 0.0;
+      x[m - 1] = x1;
+#pragma unroll 4
+      for (int r = m - 2; r >= 0; --r) {
+        const double v = (x[r] - du2[r] * x2 - du[r] * x1) * rd[r];
+        x[r] = v;
+        x2 = x1;
+        x1 = v;
+      }
+    }
+    __syncwarp();
     double mx = 0.0;
-    for (int r = 0; r < m; ++r) mx = fmax(mx, fabs(x[r]));
+    for (int r = lane; r < m; r += 32) mx = fmax(mx, fabs(x[r]));
+    mx = tri_warp_max(mx);
     double inv = mx > 0 ? 1.0 / mx : 0.0;
     double nrm = 0.0;
-    for (int r = 0; r < m; ++r) {
-      x[r] *= inv;
-      nrm += x[r] * x[r];
+    for (int r = lane; r < m; r += 32) {
+      const double v = x[r] * inv;
+      x[r] = v;
+      nrm += v * v;
     }
+    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
     inv = nrm > 0 ? 1.0 / sqrt(nrm) : 0.0;
-    for (int r = 0; r < m; ++r) x[r] *= inv;
+    for (int r = lane; r < m; r += 32) x[r] *= inv;
+    __syncwarp();
   }
-  int big = 0;
-  for (int r = 1; r < m; ++r)
-    if (fabs(x[r]) > fabs(x[big])) big = r;
-  double sg = x[big] < 0 ? -1.0 : 1.0;
-  for (int r = 0; r < m; ++r) s[r] = sg * x[r];
+  // first entry of the largest magnitude positive
+  double big = -1.0;
+  int at = 0;
+  for (int r = lane; r < m; r += 32)
+    if (fabs(x[r]) > big) big = fabs(x[r]), at = r;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, big, o);
+    const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+    if (ob > big || (ob == big && oa < at)) big = ob, at = oa;
+  }
+  const double sg = x[at] < 0 ? -1.0 : 1.0;
+  for (int r = lane; r < m; r += 32) s[r] = sg * x[r];
+}
+
+// Eigenpair i of T (alpha[0..m), beta[1..m)): theta[i] and S[i*ldS + j], one
+// warp.  The scratch is the launch's shared memory (tri_smem(m) bytes) or, for
+// matrices too large for it, `work` (6 * ldS doubles per pair).
+__device__ inline void tri_pair_one(const double* __restrict__ a, const double* __restrict__ b, int m, int i,
+                                    double* __restrict__ theta, double* __restrict__ S, int ldS,
+                                    double* __restrict__ work, double* shm) {
+  double* wk = m <= kTriSmemRows ? shm : work + (size_t)i * 6 * ldS;
+  const double th = tri_eig_one(a, b, m, i, reinterpret_cast<double2*>(wk));
+  if (threadIdx.x == 0) theta[i] = th;
+  tri_vec_one(a, b, m, th, i, wk, S + (size_t)i * ldS);
 }
 
 // Orthogonalise eigenvectors of (nearly) equal eigenvalues in order, then

@@ -77,3 +77,22 @@ def test_basis_longer_than_one_launch(env):
         assert np.all(np.abs(ev - ref[:30]) <= 1e-11 * np.max(np.abs(ref))), np.max(np.abs(ev - ref[:30]))
     finally:
         ed.ed_sector_destroy(sec)
+
+
+@pytest.mark.parametrize("power", [-20, 0, 40])
+def test_tridiagonal_solver_scales(env, power):
+    """The tridiagonal eigensolver scales its matrix by a power of two: the
+    spectrum of 2^p H is 2^p times that of H, for p of both signs (whole Krylov
+    space, so nothing depends on the residual tolerance)."""
+    ed, ctx, torch = env
+    m = W.aim(6, seed=3)
+    H = osec.build_csr(m, 3, 2)
+    ref = np.linalg.eigvalsh(H.toarray())[:6] * 2.0 ** power
+    m.T, m.U_site = m.T * 2.0 ** power, m.U_site * 2.0 ** power
+    sec = ed.ed_sector_create(ctx, m, 3, 2, "fp64")
+    try:
+        ev, _, _ = ed.ed_lanczos(sec, k=6, tol=1e-300, max_iter=H.shape[0], check_every=H.shape[0],
+                                 allow_not_converged=True)
+        assert np.all(np.abs(ev - ref) <= 1e-12 * np.max(np.abs(ref))), ev - ref
+    finally:
+        ed.ed_sector_destroy(sec)
