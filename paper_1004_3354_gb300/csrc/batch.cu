@@ -18,8 +18,9 @@
 #include <vector>
 
 #include "apply_common.h"
+#include "cgs_tile.h"
 #include "tri_common.h"
-#include "vec16.h"
+#include "vec_ops.h"
 
 struct ed_batch;
 
@@ -40,7 +41,7 @@ uint32_t default_chunk(const std::vector<uint64_t>& dims, int sms) {
   return 256;
 }
 constexpr int kBT = 256;           // threads per block
-constexpr int kKB = 8;             // basis vectors per multi-dot register group
+static_assert(kBT == kCgsThreads, "the projection tiles are shaped for one block size");
 
 struct JobDev {
   SectorView S;
@@ -64,13 +65,13 @@ struct BatchDev {
   int ms;              // coefficient row length per job (max_iter + 2)
   double* alpha;       // [job][ms]
   double* beta;
-  double* nal_d;
-  float2* nal_f;
-  double* nbe_d;
-  float2* nbe_f;
-  double* inv_d;
+  double* inv;         // 1 / beta (0 where beta vanished)
+  double* h;           // [job][ms] negated CGS projections
+  // double-float copies for the vector kernels (a conversion per thread costs
+  // more FP64 time than the element work of a small item)
+  float2* nal_f;       // -alpha
+  float2* nbe_f;       // -beta
   float2* inv_f;
-  double* h_d;         // [job][ms] negated CGS projections
   float2* h_f;
   double* scale;       // [job]
   int* exhausted;      // [job]
@@ -78,63 +79,28 @@ struct BatchDev {
   double thr;
 };
 
-template <class V>
-struct BAcc;
-template <>
-struct BAcc<double> { using T = double; };
-template <>
-struct BAcc<float2> { using T = float2; };
-template <>
-struct BAcc<float> { using T = float2; };
-
-__device__ __forceinline__ void bmac(double& a, double x, double y) { a = fma(x, y, a); }
-__device__ __forceinline__ void bmac(float2& a, float2 x, float2 y) { df_mac(a, x, y); }
-__device__ __forceinline__ void bmac(float2& a, float x, float y) { df_mac1(a, make_float2(x, 0.f), y); }
-__device__ __forceinline__ double badd(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 badd(float2 a, float2 b) { return df_add(a, b); }
-__device__ __forceinline__ double bshfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ float2 bshfl(float2 v, int o) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-__device__ __forceinline__ double bd(double a) { return a; }
-__device__ __forceinline__ double bd(float2 a) { return (double)a.x + (double)a.y; }
-__device__ __forceinline__ double bacc_of(double x) { return x; }
-__device__ __forceinline__ float2 bacc_of(float2 x) { return x; }
-__device__ __forceinline__ float2 bacc_of(float x) { return make_float2(x, 0.f); }
-__device__ __forceinline__ void bcmac(double& a, const double* cd, const float2*, size_t k, double x) {
-  a = fma(cd[k], x, a);
-}
-__device__ __forceinline__ void bcmac(float2& a, const double*, const float2* cf, size_t k, float2 x) {
-  df_mac(a, cf[k], x);
-}
-__device__ __forceinline__ void bcmac(float2& a, const double*, const float2* cf, size_t k, float x) {
-  df_mac1(a, cf[k], x);
-}
-__device__ __forceinline__ double bstore(double a, double*) { return a; }
-__device__ __forceinline__ float2 bstore(float2 a, float2*) { return df_norm(a); }
-__device__ __forceinline__ float bstore(float2 a, float*) { return __fadd_rn(a.x, a.y); }
-
 template <class A>
 __device__ __forceinline__ A bblock_sum(A v) {
   __shared__ A sh[kBT / 32];
-  for (int o = 16; o > 0; o >>= 1) v = badd(v, bshfl(v, o));
+  for (int o = 16; o > 0; o >>= 1) v = add_acc(v, shfl_x(v, o));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __syncthreads();
   if (lane == 0) sh[w] = v;
   __syncthreads();
   if (w == 0) {
     v = (lane < kBT / 32) ? sh[lane] : A{};
-    for (int o = 16; o > 0; o >>= 1) v = badd(v, bshfl(v, o));
+    for (int o = 16; o > 0; o >>= 1) v = add_acc(v, shfl_x(v, o));
   }
   return v;
 }
 
 // ---------------------------------------------------------------- step kernels
-// w = H V_j for every active sector.
+// w = H V_j for every active sector, with the item's partial of <V_j, w>.
 template <class P>
 __global__ void __launch_bounds__(kBT) k_b_apply(BatchDev B, const typename P::V* __restrict__ Vb,
                                                  typename P::V* __restrict__ w) {
   using V = typename P::V;
+  using A = typename AccOf<V>::T;
   const int j = *B.step;
   for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const uint2 item = B.items[it];
@@ -144,132 +110,113 @@ __global__ void __launch_bounds__(kBT) k_b_apply(BatchDev B, const typename P::V
     V* y = w + J.off;
     const uint32_t Dd = J.S.D_dn;
     const uint64_t e1 = min((uint64_t)item.y + B.chunk, J.dim);
+    A acc{};
     for (uint64_t e = item.y + threadIdx.x; e < e1; e += kBT) {
       const uint32_t u = (uint32_t)(e / Dd), d = (uint32_t)(e % Dd);
       const V* xr = x + (uint64_t)u * Dd;
       auto xrow = [xr](uint32_t q) { return xr[q]; };
-      y[e] = element<P>(J.S, x, u, J.ub[u], d, J.db[d], row_e<P>(J.S, u), xrow);
+      const V ye = element<P>(J.S, x, u, J.ub[u], d, J.db[d], row_e<P>(J.S, u), xrow);
+      y[e] = ye;
+      dmac(acc, xr[d], ye);
     }
+    acc = bblock_sum(acc);
+    if (threadIdx.x == 0) B.partial[it] = to_d(acc);
   }
 }
 
-// partial[slot * n_items + it] = <a, b> over the item, a/b selected by mode:
-// 0: <V_j, w>   1: <w, w>
+// partial[it] = <w, w> over the item.
 template <class V>
-__global__ void __launch_bounds__(kBT) k_b_dot(BatchDev B, const V* __restrict__ Vb, const V* __restrict__ w,
-                                               int mode) {
-  using A = typename BAcc<V>::T;
-  const int j = *B.step;
+__global__ void __launch_bounds__(kBT) k_b_norm(BatchDev B, const V* __restrict__ w) {
+  using A = typename AccOf<V>::T;
   for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const uint2 item = B.items[it];
-    if (!B.active[item.x]) continue;  // k_b_finish reads no partial of a converged sector
     A acc{};
     const JobDev& J = B.jobs[item.x];
     const uint64_t e1 = min((uint64_t)item.y + B.chunk, J.dim);
-    const V* a = (mode == 0) ? Vb + (uint64_t)j * B.tot + J.off : w + J.off;
-    const V* b = w + J.off;
-    for (uint64_t e = item.y + threadIdx.x; e < e1; e += kBT) bmac(acc, a[e], b[e]);
+    const V* a = w + J.off;
+    for (uint64_t e = item.y + threadIdx.x; e < e1; e += kBT) dmac(acc, a[e], a[e]);
     acc = bblock_sum(acc);
-    if (threadIdx.x == 0) B.partial[it] = bd(acc);
+    if (threadIdx.x == 0) B.partial[it] = to_d(acc);
   }
 }
 
-// The CGS2 kernels read sixteen-byte vectors (vec16.h).  Vector slots and
-// sector offsets are padded to 32 elements and work items start at multiples
-// of the chunk, so every item starts 16-byte aligned.
+// the negated coefficient: -d[k], or f[k], which holds it negated
+__device__ __forceinline__ void h_neg(double& o, const double* d, const float2*, size_t k) { o = -d[k]; }
+__device__ __forceinline__ void h_neg(float2& o, const double*, const float2* f, size_t k) { o = f[k]; }
 
-// Block sums of up to kKB accumulators with one barrier: each warp reduces
-// every accumulator (butterfly), then warp q reduces accumulator q over the
-// warps in the same butterfly order as bblock_sum; lane 0 of warp q stores it.
-template <class A>
-__device__ __forceinline__ void bblock_sum_group(A (&acc)[kKB], int nq, double* out, uint64_t stride) {
-  __shared__ A sh[kKB][kBT / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();  // the previous group's readers are done with sh
-#pragma unroll
-  for (int q = 0; q < kKB; ++q) {
-    A v = acc[q];
-    for (int o = 16; o > 0; o >>= 1) v = badd(v, bshfl(v, o));
-    if (lane == 0) sh[q][w] = v;
-  }
-  __syncthreads();
-  static_assert(kBT / 32 >= kKB, "one warp per accumulator");
-  if (w < nq) {
-    A v = (lane < kBT / 32) ? sh[w][lane] : A{};
-    for (int o = 16; o > 0; o >>= 1) v = badd(v, bshfl(v, o));
-    if (lane == 0) out[(uint64_t)w * stride] = bd(v);
-  }
-}
-
-// partial[k * n_items + it] = <V_k, w>, k <= j.  Sixteen-byte loads keep
-// (kKB + 1) x 16 bytes per thread in flight; the item's ragged tail (fewer
-// than one vector) is read element by element.
-template <class V>
-__global__ void __launch_bounds__(kBT) k_b_multidot(BatchDev B, const V* __restrict__ Vb, const V* __restrict__ w) {
-  using A = typename BAcc<V>::T;
-  using W16 = Vec16<V>;
-  using VT = typename W16::T;
-  constexpr int N = W16::N;
+// Projections of every active sector (cgs_tile.h), one work item per block and
+// turn: LZ the three-term update w -= alpha_j V_j + beta_j V_{j-1}; DOT the
+// partials partial[k * n_items + it] of <V_k, w>, k0 <= k < k0 + kn; UPD w +=
+// sum_k h_k V_k over the same k; UPD without DOT also the item's partial of
+// <w, w> in row 0.  A range holds at most kCgsMaxVec vectors.  Vector slots and
+// sector offsets are padded to 32 elements and items start at multiples of the
+// chunk, so every tile starts 16-byte aligned.
+template <class V, bool UPD, bool DOT, bool LZ>
+__global__ void __launch_bounds__(kBT, 2) k_b_cgs(BatchDev B, const V* __restrict__ Vb, V* __restrict__ w, int k0,
+                                                  int kn) {
+  using A = typename AccOf<V>::T;
+  constexpr uint32_t E = CgsTile<V>::E;
+  extern __shared__ __align__(16) unsigned char sm[];
+  V* wt = reinterpret_cast<V*>(sm);
+  A* hs = reinterpret_cast<A*>(sm + (DOT ? 2 * E * sizeof(V) : 0));
+  A* hsum = hs + (UPD ? kn : 0);
+  const uint32_t t = threadIdx.x;
   const int j = *B.step;
+  const int nvec = min(kn, j + 1 - k0);
+  if (nvec <= 0) return;
   for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const uint2 item = B.items[it];
-    if (!B.active[item.x]) continue;  // k_b_finish reads no partial of a converged sector
+    if (!B.active[item.x]) continue;   // the finishing kernels read no partial of a converged sector
     const JobDev& J = B.jobs[item.x];
-    const uint64_t e0 = J.off + item.y;
-    const uint64_t n = min((uint64_t)item.y + B.chunk, J.dim) - item.y;
-    const uint64_t nv = n / N;
-    const VT* wv = reinterpret_cast<const VT*>(w + e0);
-    for (int k0 = 0; k0 <= j; k0 += kKB) {
-      const int nq = min(kKB, j + 1 - k0);
-      A acc[kKB];
-#pragma unroll
-      for (int q = 0; q < kKB; ++q) acc[q] = A{};
-      {
-        const V* vk = Vb + (uint64_t)k0 * B.tot + e0;
-        for (uint64_t t = threadIdx.x; t < nv; t += kBT) {
-          const VT wq = wv[t];
-          VT vq[kKB];
-#pragma unroll
-          for (int q = 0; q < kKB; ++q)
-            if (q < nq) vq[q] = __ldg(reinterpret_cast<const VT*>(vk + (uint64_t)q * B.tot) + t);
-#pragma unroll
-          for (int q = 0; q < kKB; ++q)
-            if (q < nq) {
-#pragma unroll
-              for (int i = 0; i < N; ++i) bmac(acc[q], W16::get(vq[q], i), W16::get(wq, i));
-            }
-        }
-        for (uint64_t e = nv * N + threadIdx.x; e < n; e += kBT) {
-          const V we = w[e0 + e];
-#pragma unroll
-          for (int q = 0; q < kKB; ++q)
-            if (q < nq) bmac(acc[q], vk[(uint64_t)q * B.tot + e], we);
-        }
-      }
-      bblock_sum_group(acc, nq, B.partial + (uint64_t)k0 * B.n_items + it, B.n_items);
+    const size_t base = (size_t)item.x * B.ms;
+    __syncthreads();   // the previous item's sums are written
+    if (UPD)
+      for (int k = t; k < nvec; k += kBT) h_pick(hs[k], B.h, B.h_f, base + k0 + k);
+    if (DOT)
+      for (int k = t; k < nvec; k += kBT) hsum[k] = A{};
+    A na{}, nb{};
+    if (LZ) {
+      h_neg(na, B.alpha, B.nal_f, base + j);
+      h_neg(nb, B.beta, B.nbe_f, base + j);
+    }
+    __syncthreads();
+    const uint32_t n = (uint32_t)(min((uint64_t)item.y + B.chunk, J.dim) - item.y);
+    const uint64_t g0 = J.off + item.y;
+    A nacc{};
+    int buf = 0;
+    for (uint32_t e = 0; e < n; e += E, buf ^= 1) {
+      const V* vt = Vb + (uint64_t)k0 * B.tot + g0 + e;
+      const V* vj = Vb + (uint64_t)j * B.tot + g0 + e;
+      cgs_tile<V, UPD, DOT, A>(vt, B.tot, nvec, w + g0 + e, min(E, n - e), hs, hsum, wt + buf * E,
+                               LZ ? vj : nullptr, LZ && j > 0 ? vj - B.tot : nullptr, na, nb, nacc);
+    }
+    if (DOT) {
+      __syncthreads();
+      for (int k = t; k < nvec; k += kBT) B.partial[(uint64_t)(k0 + k) * B.n_items + it] = to_d(hsum[k]);
+    }
+    if (UPD && !DOT) {
+      nacc = bblock_sum(nacc);
+      if (t == 0) B.partial[it] = to_d(nacc);
     }
   }
 }
 
-enum { BF_ALPHA = 0, BF_BETA = 1, BF_NEGH = 2, BF_NORM0 = 3 };
+enum { BF_ALPHA, BF_BETA, BF_NORM0 };
 
-// One block per (job, k): sum the job's item partials of row k and store.
+// One block per job: sum the job's item partials (row 0) and store.
 __global__ void __launch_bounds__(kBT) k_b_finish(BatchDev B, int op) {
-  const int job = blockIdx.x, k = blockIdx.y;
+  const int job = blockIdx.x;
   const int j = *B.step;
   if (!B.active[job]) return;
-  if (op == BF_NEGH && k > j) return;
   const JobDev& J = B.jobs[job];
-  const int row = (op == BF_NEGH) ? k : 0;
   double v = 0.0;
-  for (uint32_t it = J.item0 + threadIdx.x; it < J.item1; it += kBT) v += B.partial[(uint64_t)row * B.n_items + it];
+  for (uint32_t it = J.item0 + threadIdx.x; it < J.item1; it += kBT) v += B.partial[it];
   v = bblock_sum(v);
   if (threadIdx.x != 0) return;
   const size_t base = (size_t)job * B.ms;
   switch (op) {
     case BF_ALPHA:
       B.alpha[base + j] = v;
-      B.nal_d[base + j] = -v;
       B.nal_f[base + j] = df_from_double(-v);
       B.scale[job] = fmax(B.scale[job], fabs(v));
       break;
@@ -279,22 +226,17 @@ __global__ void __launch_bounds__(kBT) k_b_finish(BatchDev B, int op) {
       B.scale[job] = sc;
       const bool dead = !(b > B.thr * fmax(sc, 1.0));
       if (dead && B.exhausted[job] < 0) B.exhausted[job] = j + 1;
-      B.beta[base + j + 1] = dead ? 0.0 : b;
-      B.nbe_d[base + j + 1] = dead ? 0.0 : -b;
-      B.nbe_f[base + j + 1] = df_from_double(dead ? 0.0 : -b);
       const double inv = dead ? 0.0 : 1.0 / b;
-      B.inv_d[base + j + 1] = inv;
+      B.beta[base + j + 1] = dead ? 0.0 : b;
+      B.nbe_f[base + j + 1] = df_from_double(dead ? 0.0 : -b);
+      B.inv[base + j + 1] = inv;
       B.inv_f[base + j + 1] = df_from_double(inv);
       break;
     }
-    case BF_NEGH:
-      B.h_d[base + k] = -v;
-      B.h_f[base + k] = df_from_double(-v);
-      break;
     case BF_NORM0: {
       const double b = sqrt(fmax(v, 0.0));
       const double inv = b > 0.0 ? 1.0 / b : 0.0;
-      B.inv_d[base] = inv;
+      B.inv[base] = inv;
       B.inv_f[base] = df_from_double(inv);
       B.beta[base] = 0.0;
       break;
@@ -302,75 +244,45 @@ __global__ void __launch_bounds__(kBT) k_b_finish(BatchDev B, int op) {
   }
 }
 
-// mode 0: w += nal_j V_j + nbe_j V_{j-1}
-// mode 2: V_{j+1} = inv_{j+1} w        mode 3: V_0 = inv_0 w
-template <class V>
-__global__ void __launch_bounds__(kBT) k_b_axpy(BatchDev B, V* __restrict__ Vb, V* __restrict__ w, int mode) {
-  using A = typename BAcc<V>::T;
+// Negated projections h_k, k <= j, of every job: one warp per (job, k), a fixed
+// grid of kHWarps warps per job (a block per possible k would launch ms blocks
+// per job, most of them with nothing to do).
+constexpr int kHWarps = 64;
+__global__ void __launch_bounds__(kBT) k_b_finish_h(BatchDev B) {
+  const int job = blockIdx.x;
   const int j = *B.step;
-  for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
-    const uint2 item = B.items[it];
-    if (!B.active[item.x]) continue;
-    const JobDev& J = B.jobs[item.x];
-    const size_t base = (size_t)item.x * B.ms;
-    const uint64_t e1 = min((uint64_t)item.y + B.chunk, J.dim);
-    for (uint64_t e = item.y + threadIdx.x; e < e1; e += kBT) {
-      const uint64_t g = J.off + e;
-      if (mode == 0) {
-        A a = bacc_of(w[g]);
-        bcmac(a, B.nal_d, B.nal_f, base + j, Vb[(uint64_t)j * B.tot + g]);
-        if (j > 0) bcmac(a, B.nbe_d, B.nbe_f, base + j, Vb[(uint64_t)(j - 1) * B.tot + g]);
-        w[g] = bstore(a, w);
-      } else {
-        const int s = (mode == 2) ? j + 1 : 0;
-        A a{};
-        bcmac(a, B.inv_d, B.inv_f, base + s, w[g]);
-        Vb[(uint64_t)s * B.tot + g] = bstore(a, Vb);
-      }
+  if (!B.active[job]) return;
+  const JobDev& J = B.jobs[job];
+  const int lane = threadIdx.x & 31;
+  for (int k = blockIdx.y * (kBT / 32) + (threadIdx.x >> 5); k <= j; k += kHWarps) {
+    double v = 0.0;
+    const double* p = B.partial + (uint64_t)k * B.n_items;
+    for (uint32_t it = J.item0 + lane; it < J.item1; it += 32) v += p[it];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) {
+      B.h[(size_t)job * B.ms + k] = -v;
+      B.h_f[(size_t)job * B.ms + k] = df_from_double(-v);
     }
   }
 }
 
-// CGS2 update w += sum_{k<=j} h_k V_k for every active sector: sixteen-byte
-// loads of w and of each V_k, each element's terms in the order k = 0..j
-// (the ragged tail of an item element by element).
+// V_s = inv_s w with s = j + 1 (a step) or 0 (the start vector).
 template <class V>
-__global__ void __launch_bounds__(kBT) k_b_cgs_update(BatchDev B, const V* __restrict__ Vb, V* __restrict__ w) {
-  using A = typename BAcc<V>::T;
-  using W16 = Vec16<V>;
-  using VT = typename W16::T;
-  constexpr int N = W16::N;
-  const int j = *B.step;
+__global__ void __launch_bounds__(kBT) k_b_scale(BatchDev B, V* __restrict__ Vb, const V* __restrict__ w, int start) {
+  using A = typename AccOf<V>::T;
+  const int s = start ? 0 : *B.step + 1;
   for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const uint2 item = B.items[it];
     if (!B.active[item.x]) continue;
     const JobDev& J = B.jobs[item.x];
-    const size_t base = (size_t)item.x * B.ms;
-    const uint64_t e0 = J.off + item.y;
-    const uint64_t n = min((uint64_t)item.y + B.chunk, J.dim) - item.y;
-    const uint64_t nv = n / N;
-    VT* wv = reinterpret_cast<VT*>(w + e0);
-    const V* v0 = Vb + e0;
-    for (uint64_t t = threadIdx.x; t < nv; t += kBT) {
-      const VT wq = wv[t];
-      A a[N];
-#pragma unroll
-      for (int i = 0; i < N; ++i) a[i] = bacc_of(W16::get(wq, i));
-#pragma unroll 4
-      for (int k = 0; k <= j; ++k) {
-        const VT vq = __ldg(reinterpret_cast<const VT*>(v0 + (uint64_t)k * B.tot) + t);
-#pragma unroll
-        for (int i = 0; i < N; ++i) bcmac(a[i], B.h_d, B.h_f, base + k, W16::get(vq, i));
-      }
-      VT o;
-#pragma unroll
-      for (int i = 0; i < N; ++i) W16::set(o, i, bstore(a[i], w));
-      wv[t] = o;
-    }
-    for (uint64_t e = nv * N + threadIdx.x; e < n; e += kBT) {
-      A a = bacc_of(w[e0 + e]);
-      for (int k = 0; k <= j; ++k) bcmac(a, B.h_d, B.h_f, base + k, v0[(uint64_t)k * B.tot + e]);
-      w[e0 + e] = bstore(a, w);
+    A c;
+    h_pick(c, B.inv, B.inv_f, (size_t)item.x * B.ms + s);
+    const uint64_t e1 = min((uint64_t)item.y + B.chunk, J.dim);
+    for (uint64_t e = item.y + threadIdx.x; e < e1; e += kBT) {
+      const uint64_t g = J.off + e;
+      A a{};
+      hmac(a, c, w[g]);
+      Vb[(uint64_t)s * B.tot + g] = store_v(a, Vb);
     }
   }
 }
@@ -406,15 +318,12 @@ __global__ void k_b_random(BatchDev B, V* __restrict__ w, uint64_t seed) {
 __device__ __forceinline__ void rmac(double& a, double s, float2, double v) { a = fma(s, v, a); }
 __device__ __forceinline__ void rmac(float2& a, double, float2 s, float2 v) { df_mac(a, s, v); }
 __device__ __forceinline__ void rmac(float2& a, double, float2 s, float v) { df_mac1(a, s, v); }
-__device__ __forceinline__ double rout(double a, double*) { return a; }
-__device__ __forceinline__ float2 rout(float2 a, float2*) { return df_norm(a); }
-__device__ __forceinline__ float rout(float2 a, float*) { return __fadd_rn(a.x, a.y); }
 
 template <class V>
 __global__ void k_b_ritz(BatchDev B, const V* __restrict__ Vb, const double* __restrict__ S,
                          const float2* __restrict__ Sf, const int* __restrict__ mj, const int* __restrict__ kj,
                          int kmax, V* const* __restrict__ outs) {
-  using A = typename BAcc<V>::T;
+  using A = typename AccOf<V>::T;
   for (uint32_t it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const uint2 item = B.items[it];
     V* out = outs[item.x];
@@ -427,7 +336,7 @@ __global__ void k_b_ritz(BatchDev B, const V* __restrict__ Vb, const double* __r
         const size_t row = ((size_t)item.x * kmax + i) * B.ms;
         A acc{};
         for (int j = 0; j < m; ++j) rmac(acc, S[row + j], Sf[row + j], Vb[(uint64_t)j * B.tot + J.off + e]);
-        out[(uint64_t)i * J.dim + e] = rout(acc, out);
+        out[(uint64_t)i * J.dim + e] = store_v(acc, out);
       }
   }
 }
@@ -564,13 +473,11 @@ int batch_run(Batch* bt, const ed_lanczos_opts* o, double* evals, int* iters, ed
   ED_TRY(R.alloc(&B.step, 1));
   ED_TRY(R.alloc(&B.alpha, (size_t)J * ms));
   ED_TRY(R.alloc(&B.beta, (size_t)J * ms));
-  ED_TRY(R.alloc(&B.nal_d, (size_t)J * ms));
+  ED_TRY(R.alloc(&B.inv, (size_t)J * ms));
+  ED_TRY(R.alloc(&B.h, (size_t)J * ms));
   ED_TRY(R.alloc(&B.nal_f, (size_t)J * ms));
-  ED_TRY(R.alloc(&B.nbe_d, (size_t)J * ms));
   ED_TRY(R.alloc(&B.nbe_f, (size_t)J * ms));
-  ED_TRY(R.alloc(&B.inv_d, (size_t)J * ms));
   ED_TRY(R.alloc(&B.inv_f, (size_t)J * ms));
-  ED_TRY(R.alloc(&B.h_d, (size_t)J * ms));
   ED_TRY(R.alloc(&B.h_f, (size_t)J * ms));
   ED_TRY(R.alloc(&B.scale, J));
   ED_TRY(R.alloc(&B.exhausted, J));
@@ -590,8 +497,6 @@ int batch_run(Batch* bt, const ed_lanczos_opts* o, double* evals, int* iters, ed
 
   ED_TRY_CUDA(cudaMemsetAsync(B.alpha, 0, sizeof(double) * J * ms, st));
   ED_TRY_CUDA(cudaMemsetAsync(B.beta, 0, sizeof(double) * J * ms, st));
-  ED_TRY_CUDA(cudaMemsetAsync(B.nbe_d, 0, sizeof(double) * J * ms, st));
-  ED_TRY_CUDA(cudaMemsetAsync(B.nbe_f, 0, sizeof(float2) * J * ms, st));
   ED_TRY_CUDA(cudaMemsetAsync(B.scale, 0, sizeof(double) * J, st));
   ED_TRY_CUDA(cudaMemsetAsync(B.exhausted, 0xff, sizeof(int) * J, st));  // -1
   ED_TRY_CUDA(cudaMemsetAsync(B.step, 0, sizeof(int), st));
@@ -601,12 +506,12 @@ int batch_run(Batch* bt, const ed_lanczos_opts* o, double* evals, int* iters, ed
   ED_TRY_CUDA(cudaMemcpyAsync(dk, h_k.data(), sizeof(int) * J, cudaMemcpyHostToDevice, st));
 
   const uint32_t grid = (uint32_t)std::min<uint64_t>(B.n_items, (uint64_t)ctx->num_sms * 8);
-  const dim3 fgrid(J, 1), hgrid(J, ms);
+  const dim3 hgrid(J, kHWarps / (kBT / 32));
   // start vectors: random, normalised per sector
   k_b_random<V><<<grid, kBT, 0, st>>>(B, w, o->seed);
-  k_b_dot<V><<<grid, kBT, 0, st>>>(B, Vb, w, 1);
-  k_b_finish<<<fgrid, kBT, 0, st>>>(B, BF_NORM0);
-  k_b_axpy<V><<<grid, kBT, 0, st>>>(B, Vb, w, 3);
+  k_b_norm<V><<<grid, kBT, 0, st>>>(B, w);
+  k_b_finish<<<J, kBT, 0, st>>>(B, BF_NORM0);
+  k_b_scale<V><<<grid, kBT, 0, st>>>(B, Vb, w, 1);
   ED_LAUNCH_CHECK();
 
   // one Lanczos step for all active sectors, captured once
@@ -614,17 +519,31 @@ int batch_run(Batch* bt, const ed_lanczos_opts* o, double* evals, int* iters, ed
   cudaGraphExec_t exec = nullptr;
   ED_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   k_b_apply<P><<<grid, kBT, 0, st>>>(B, Vb, w);
-  k_b_dot<V><<<grid, kBT, 0, st>>>(B, Vb, w, 0);
-  k_b_finish<<<fgrid, kBT, 0, st>>>(B, BF_ALPHA);
-  k_b_axpy<V><<<grid, kBT, 0, st>>>(B, Vb, w, 0);
-  for (int pass = 0; pass < 2; ++pass) {
-    k_b_multidot<V><<<grid, kBT, 0, st>>>(B, Vb, w);
-    k_b_finish<<<hgrid, kBT, 0, st>>>(B, BF_NEGH);
-    k_b_cgs_update<V><<<grid, kBT, 0, st>>>(B, Vb, w);
+  k_b_finish<<<J, kBT, 0, st>>>(B, BF_ALPHA);
+  if (mmax <= kCgsMaxVec) {
+    // three sweeps over the bases: the first update and the second projection share one
+    k_b_cgs<V, false, true, true><<<grid, kBT, cgs_smem<V>(mmax, false, true), st>>>(B, Vb, w, 0, mmax);
+    k_b_finish_h<<<hgrid, kBT, 0, st>>>(B);
+    k_b_cgs<V, true, true, false><<<grid, kBT, cgs_smem<V>(mmax, true, true), st>>>(B, Vb, w, 0, mmax);
+    k_b_finish_h<<<hgrid, kBT, 0, st>>>(B);
+    k_b_cgs<V, true, false, false><<<grid, kBT, cgs_smem<V>(mmax, true, false), st>>>(B, Vb, w, 0, mmax);
+  } else {   // more vectors than a block's shared memory serves at once: range by range
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int k0 = 0; k0 < mmax; k0 += kCgsMaxVec) {
+        const int kn = std::min(kCgsMaxVec, mmax - k0);
+        const size_t sb = cgs_smem<V>(kn, false, true);
+        if (pass == 0 && k0 == 0) k_b_cgs<V, false, true, true><<<grid, kBT, sb, st>>>(B, Vb, w, k0, kn);
+        else k_b_cgs<V, false, true, false><<<grid, kBT, sb, st>>>(B, Vb, w, k0, kn);
+      }
+      k_b_finish_h<<<hgrid, kBT, 0, st>>>(B);
+      for (int k0 = 0; k0 < mmax; k0 += kCgsMaxVec) {
+        const int kn = std::min(kCgsMaxVec, mmax - k0);
+        k_b_cgs<V, true, false, false><<<grid, kBT, cgs_smem<V>(kn, true, false), st>>>(B, Vb, w, k0, kn);
+      }
+    }
   }
-  k_b_dot<V><<<grid, kBT, 0, st>>>(B, Vb, w, 1);
-  k_b_finish<<<fgrid, kBT, 0, st>>>(B, BF_BETA);
-  k_b_axpy<V><<<grid, kBT, 0, st>>>(B, Vb, w, 2);
+  k_b_finish<<<J, kBT, 0, st>>>(B, BF_BETA);
+  k_b_scale<V><<<grid, kBT, 0, st>>>(B, Vb, w, 0);
   k_b_step_inc<<<1, 1, 0, st>>>(B.step);
   cudaError_t ce = cudaStreamEndCapture(st, &graph);
   if (ce != cudaSuccess) {

@@ -42,6 +42,10 @@ struct CgsTile {
 __device__ __forceinline__ void h_split(double& o, double h) { o = h; }
 __device__ __forceinline__ void h_split(float2& o, double h) { o = df_from_double(h); }
 
+// coefficient k in the accumulator's format, from its double or double-float copy
+__device__ __forceinline__ void h_pick(double& o, const double* d, const float2*, size_t k) { o = d[k]; }
+__device__ __forceinline__ void h_pick(float2& o, const double*, const float2* f, size_t k) { o = f[k]; }
+
 // a += h * x, h in the accumulator's format
 __device__ __forceinline__ void hmac(double& a, double h, double x) { a = fma(h, x, a); }
 __device__ __forceinline__ void hmac(float2& a, float2 h, float2 x) { df_mac(a, h, x); }
@@ -112,14 +116,21 @@ __device__ __forceinline__ void tile_dots(const V* __restrict__ vt, uint64_t str
         if (full) {
 #pragma unroll
           for (int i = 0; i < NV; ++i) v[i] = __ldg(reinterpret_cast<const VT*>(vk) + i * 32 + lane);
+#pragma unroll
+          for (int i = 0; i < NV; ++i)
+#pragma unroll
+            for (int c = 0; c < N; ++c) dmac(acc[q], W16::get(v[i], c), W16::get(wq[i], c));
         } else {
 #pragma unroll
-          for (int i = 0; i < NV; ++i) v[i] = tile_ld(vk, i * 32 + lane, lim);
+          for (int i = 0; i < NV; ++i)
+            if ((uint32_t)i * 32 * N < lim) v[i] = tile_ld(vk, i * 32 + lane, lim);
+#pragma unroll
+          for (int i = 0; i < NV; ++i)
+            if ((uint32_t)i * 32 * N < lim) {
+#pragma unroll
+              for (int c = 0; c < N; ++c) dmac(acc[q], W16::get(v[i], c), W16::get(wq[i], c));
+            }
         }
-#pragma unroll
-        for (int i = 0; i < NV; ++i)
-#pragma unroll
-          for (int c = 0; c < N; ++c) dmac(acc[q], W16::get(v[i], c), W16::get(wq[i], c));
       }
     }
     const A s = warp_sum8(acc, lane);
@@ -128,16 +139,18 @@ __device__ __forceinline__ void tile_dots(const V* __restrict__ vt, uint64_t str
   }
 }
 
-// Sum of nb doubles by the whole block, the same in every thread and block.
+// Sum of nb doubles, the same in every thread and block: the first warp sums
+// (FP64 additions of a whole block would take longer than the rest of a small
+// kernel) and the block shares the result through sh.
 __device__ __forceinline__ double block_total(const double* __restrict__ p, int nb, double* sh) {
-  double v = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) v += p[i];
-  v = block_reduce(v, sh);
-  if (threadIdx.x == 0) sh[0] = v;
+  if (threadIdx.x < 32) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < nb; i += 32) v += p[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) sh[0] = v;
+  }
   __syncthreads();
-  v = sh[0];
-  __syncthreads();
-  return v;
+  return sh[0];
 }
 
 // Three-term update w -= alpha_j v_j + beta_j v_{j-1} ahead of the first
@@ -153,56 +166,29 @@ struct LzTerm {
   double* scale = nullptr;     // running maximum of |alpha|, beta
 };
 
-// UPD: w += sum_k h_k V_k (h holds the negated projections); DOT: partials
-// hpart[k * gridDim.x + b] of <V_k, w> with the updated w; UPD without DOT:
-// partials npart[b] of <w, w>.  rev walks the tiles from the last one, so that
-// a kernel starts on what the one before it left in L2.
-template <class V, bool UPD, bool DOT>
-__global__ void __launch_bounds__(kCgsThreads, 2) k_cgs(const V* __restrict__ Vb, uint64_t stride, int nvec,
-                                                        V* __restrict__ w, uint64_t n, int rev,
-                                                        const double* __restrict__ h, double* __restrict__ hpart,
-                                                        double* __restrict__ npart, LzTerm<V> lz) {
-  using A = typename AccOf<V>::T;
+// One tile (lim elements at w0, the same elements of the basis at vt).  UPD: w
+// += sum_k hs_k V_k (hs: the negated projections); else with lv != NULL the
+// three-term update w += na lv + nb lvp.  DOT: <V_k, w> of the updated w added
+// to hsum[k], through the tile buffer wb (the caller alternates two: a warp
+// still reading one tile's buffer holds the barrier of the next tile, past
+// which the buffer is written again).  UPD without DOT: nacc += <w, w>.
+template <class V, bool UPD, bool DOT, class A>
+__device__ __forceinline__ void cgs_tile(const V* __restrict__ vt, uint64_t stride, int nvec, V* w0, uint32_t lim,
+                                         const A* hs, A* hsum, V* wb, const V* __restrict__ lv,
+                                         const V* __restrict__ lvp, A na, A nb, A& nacc) {
   using W16 = Vec16<V>;
   using VT = typename W16::T;
   constexpr int N = W16::N;
-  constexpr uint32_t E = CgsTile<V>::E;
-  extern __shared__ __align__(16) unsigned char sm[];
-  V* wt = reinterpret_cast<V*>(sm);                                   // two tiles of w
-  A* hs = reinterpret_cast<A*>(sm + (DOT ? 2 * E * sizeof(V) : 0));   // coefficients (UPD)
-  A* hsum = hs + (UPD ? nvec : 0);                                    // the block's sums (DOT)
-  __shared__ double shd[32];
-  __shared__ A sha[32];
   const uint32_t t = threadIdx.x;
-  A na{}, nb{};   // -alpha_j, -beta_j
-  if (lz.v) {
-    const double al = block_total(lz.apart, lz.na, shd);
-    h_split(na, -al);
-    if (lz.vp) h_split(nb, -*lz.beta);
-    if (blockIdx.x == 0 && t == 0) {
-      *lz.alpha = al;
-      *lz.scale = fmax(*lz.scale, fabs(al));
-    }
-  }
-  if (UPD)
-    for (int k = t; k < nvec; k += kCgsThreads) h_split(hs[k], h[k]);
-  if (DOT)
-    for (int k = t; k < nvec; k += kCgsThreads) hsum[k] = A{};
-  if (UPD || DOT) __syncthreads();
-  A nacc{};
-  const uint32_t tiles = (uint32_t)((n + E - 1) / E);
-  int buf = 0;
-  for (uint32_t ti = blockIdx.x; ti < tiles; ti += gridDim.x, buf ^= 1) {
-    const uint64_t e0 = (uint64_t)(rev ? tiles - 1 - ti : ti) * E;
-    const uint32_t lim = (uint32_t)(n - e0 < E ? n - e0 : E);
-    VT wv = tile_ld<V, false>(w + e0, t, lim);
-    if (UPD || lz.v) {
+  VT wv{};
+  if (t * N < lim) {
+    wv = tile_ld<V, false>(w0, t, lim);
+    if (UPD || lv) {
       A a[N];
 #pragma unroll
       for (int c = 0; c < N; ++c) a[c] = acc_of(W16::get(wv, c));
       if (UPD) {
-        const V* vt = Vb + e0;
-        if (lim == E) {
+        if ((t + 1) * N <= lim) {
           const VT* vp = reinterpret_cast<const VT*>(vt) + t;
           const uint64_t sv = stride / N;
           int k = 0;
@@ -221,7 +207,6 @@ __global__ void __launch_bounds__(kCgsThreads, 2) k_cgs(const V* __restrict__ Vb
             for (int c = 0; c < N; ++c) hmac(a[c], hs[k], W16::get(v, c));
           }
         } else {
-#pragma unroll 4
           for (int k = 0; k < nvec; ++k) {
             const VT v = tile_ld<V>(vt + (uint64_t)k * stride, t, lim);
 #pragma unroll
@@ -229,37 +214,83 @@ __global__ void __launch_bounds__(kCgsThreads, 2) k_cgs(const V* __restrict__ Vb
           }
         }
       } else {
-        const VT v = tile_ld<V>(lz.v + e0, t, lim);
+        const VT v = tile_ld<V>(lv, t, lim);
 #pragma unroll
         for (int c = 0; c < N; ++c) hmac(a[c], na, W16::get(v, c));
-        if (lz.vp) {
-          const VT u = tile_ld<V>(lz.vp + e0, t, lim);
+        if (lvp) {
+          const VT u = tile_ld<V>(lvp, t, lim);
 #pragma unroll
           for (int c = 0; c < N; ++c) hmac(a[c], nb, W16::get(u, c));
         }
       }
 #pragma unroll
       for (int c = 0; c < N; ++c) {
-        const V o = store_v(a[c], w);
+        const V o = store_v(a[c], w0);
         W16::set(wv, c, o);
         if (UPD && !DOT && t * N + c < lim) dmac(nacc, o, o);
       }
       if ((t + 1) * N <= lim) {
-        reinterpret_cast<VT*>(w + e0)[t] = wv;
+        reinterpret_cast<VT*>(w0)[t] = wv;
       } else {
 #pragma unroll
         for (int c = 0; c < N; ++c)
-          if (t * N + c < lim) w[e0 + t * N + c] = W16::get(wv, c);
+          if (t * N + c < lim) w0[t * N + c] = W16::get(wv, c);
       }
     }
-    if (DOT) {
-      // two buffers: a warp still reading one tile's buffer holds the barrier
-      // of the next tile, past which the buffer is written again
-      V* wb = wt + buf * E;
-      reinterpret_cast<VT*>(wb)[t] = wv;
-      __syncthreads();
-      tile_dots<V, A>(Vb + e0, stride, nvec, wb, lim, hsum);
+  }
+  if (DOT) {
+    reinterpret_cast<VT*>(wb)[t] = wv;
+    __syncthreads();
+    tile_dots<V, A>(vt, stride, nvec, wb, lim, hsum);
+  }
+}
+
+// The projection of one vector: UPD, DOT and LzTerm as in cgs_tile, with the
+// negated projections h; DOT writes the partials hpart[k * gridDim.x + b] of
+// <V_k, w>, UPD without DOT the partials npart[b] of <w, w>.  rev walks the
+// tiles from the last one, so that a kernel starts on what the one before it
+// left in L2.
+template <class V, bool UPD, bool DOT>
+__global__ void __launch_bounds__(kCgsThreads, 2) k_cgs(const V* __restrict__ Vb, uint64_t stride, int nvec,
+                                                        V* __restrict__ w, uint64_t n, int rev,
+                                                        const double* __restrict__ h, const float2* __restrict__ hf,
+                                                        double* __restrict__ hpart, double* __restrict__ npart,
+                                                        LzTerm<V> lz) {
+  using A = typename AccOf<V>::T;
+  constexpr uint32_t E = CgsTile<V>::E;
+  extern __shared__ __align__(16) unsigned char sm[];
+  V* wt = reinterpret_cast<V*>(sm);                                   // two tiles of w
+  A* hs = reinterpret_cast<A*>(sm + (DOT ? 2 * E * sizeof(V) : 0));   // coefficients (UPD)
+  A* hsum = hs + (UPD ? nvec : 0);                                    // the block's sums (DOT)
+  __shared__ double shd[32];
+  __shared__ A sha[32];
+  const uint32_t t = threadIdx.x;
+  if (lz.v) {
+    const double al = block_total(lz.apart, lz.na, shd);
+    if (t == 0) {   // one thread: FP64 arithmetic of a whole block takes a microsecond
+      h_split(sha[0], -al);
+      h_split(sha[1], lz.vp ? -*lz.beta : 0.0);
+      if (blockIdx.x == 0) {
+        *lz.alpha = al;
+        *lz.scale = fmax(*lz.scale, fabs(al));
+      }
     }
+  }
+  if (UPD)
+    for (int k = t; k < nvec; k += kCgsThreads) h_pick(hs[k], h, hf, k);
+  if (DOT)
+    for (int k = t; k < nvec; k += kCgsThreads) hsum[k] = A{};
+  __syncthreads();
+  A na{}, nb{};   // -alpha_j, -beta_j
+  if (lz.v) na = sha[0], nb = sha[1];
+  A nacc{};
+  const uint32_t tiles = (uint32_t)((n + E - 1) / E);
+  int buf = 0;
+  for (uint32_t ti = blockIdx.x; ti < tiles; ti += gridDim.x, buf ^= 1) {
+    const uint64_t e0 = (uint64_t)(rev ? tiles - 1 - ti : ti) * E;
+    const uint32_t lim = (uint32_t)(n - e0 < E ? n - e0 : E);
+    cgs_tile<V, UPD, DOT, A>(Vb + e0, stride, nvec, w + e0, lim, hs, hsum, wt + buf * E, lz.v ? lz.v + e0 : nullptr,
+                             lz.vp ? lz.vp + e0 : nullptr, na, nb, nacc);
   }
   if (DOT) {
     __syncthreads();

@@ -41,6 +41,7 @@ struct Coefs {
   double* inv_d;    // 1 / beta (0 when beta vanished)
   float2* inv_f;
   double* h_d;      // -h (CGS projections)
+  float2* h_f;
   double* scale;    // running max |alpha|, beta (two slots: k_scale_beta reads one and writes the other)
   int* exhausted;   // first step with a vanished beta, -1 if none
   double* out;      // generic scalar output slots
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict
     case OP_SUM: c.out[slot + o] = v; break;
     case OP_NEGH:
       c.h_d[slot + o] = -v;
+      c.h_f[slot + o] = df_from_double(-v);
       break;
     case OP_NORM_INV: {
       double b = sqrt(fmax(v, 0.0));
@@ -179,16 +181,21 @@ __global__ void __launch_bounds__(kRedThreads) k_scale_beta(const V* __restrict_
   using W16 = Vec16<V>;
   using VT = typename W16::T;
   __shared__ double sh[32];
-  const double b = sqrt(fmax(block_total(partial, nb, sh), 0.0));
-  const double sc = fmax(c.scale[ph], b);
-  const bool dead = !(b > thr * fmax(sc, 1.0));
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    c.scale[1 - ph] = sc;
-    if (dead && *c.exhausted < 0) *c.exhausted = slot;
-    c.beta[slot] = dead ? 0.0 : b;
+  __shared__ A inv_s;
+  const double tot = block_total(partial, nb, sh);
+  if (threadIdx.x == 0) {   // one thread: FP64 roots and divisions of a whole block would take microseconds
+    const double b = sqrt(fmax(tot, 0.0));
+    const double sc = fmax(c.scale[ph], b);
+    const bool dead = !(b > thr * fmax(sc, 1.0));
+    if (blockIdx.x == 0) {
+      c.scale[1 - ph] = sc;
+      if (dead && *c.exhausted < 0) *c.exhausted = slot;
+      c.beta[slot] = dead ? 0.0 : b;
+    }
+    h_split(inv_s, dead ? 0.0 : 1.0 / b);
   }
-  A inv;
-  h_split(inv, dead ? 0.0 : 1.0 / b);
+  __syncthreads();
+  const A inv = inv_s;
   const uint64_t nv = (n + W16::N - 1) / W16::N;
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t e0 = t * W16::N;
@@ -330,17 +337,17 @@ int cgs2(Work<V>& W, const V* Vb, uint64_t stride, int nvec, V* w, LzTerm<V> lz 
   };
   auto dots = [&](int k0, int kn, int rev, const LzTerm<V>& t) {
     k_cgs<V, false, true><<<nb, kCgsThreads, cgs_smem<V>(kn, false, true), W.st>>>(
-        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, nullptr, W.hpart, nullptr, t);
+        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, nullptr, nullptr, W.hpart, nullptr, t);
     finish(k0, kn);
   };
   auto update = [&](int k0, int kn, int rev) {
     k_cgs<V, true, false><<<nb, kCgsThreads, cgs_smem<V>(kn, true, false), W.st>>>(
-        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, W.c.h_d + k0, nullptr, W.partial, none);
+        Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, W.c.h_d + k0, W.c.h_f + k0, nullptr, W.partial, none);
   };
   if (nvec <= kCgsMaxVec) {
     dots(0, nvec, 0, lz);
     k_cgs<V, true, true><<<nb, kCgsThreads, cgs_smem<V>(nvec, true, true), W.st>>>(
-        Vb, stride, nvec, w, W.n, 1, W.c.h_d, W.hpart, nullptr, none);
+        Vb, stride, nvec, w, W.n, 1, W.c.h_d, W.c.h_f, W.hpart, nullptr, none);
     finish(0, nvec);
     update(0, nvec, 0);
   } else {   // a basis of more vectors than a block's shared memory serves at once: range by range
@@ -392,7 +399,7 @@ int lanczos_step(const Sector* s, Work<V>& W, const V* Vb, uint64_t ld, int j, c
   lz.scale = W.c.scale + W.ph;
   ED_TRY(cgs2(W, Vb, ld, j + 1, w, lz));
   const uint32_t grid =
-      (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((W.n / Vec16<V>::N + 255) / 256, (uint64_t)W.ctx->num_sms * 8));
+      (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((W.n / Vec16<V>::N + 255) / 256, (uint64_t)W.ctx->num_sms * 4));
   k_scale_beta<V><<<grid, kRedThreads, 0, W.st>>>(w, vnext, W.n, W.partial, (int)cgs_grid<V>(W.ctx, W.n), W.c, j + 1,
                                                  W.ph, thr);
   ED_LAUNCH_CHECK();
@@ -440,6 +447,7 @@ Coefs carve_coefs(Carve& cv, int mmax) {
   c.inv_d = cv.take<double>(m2);
   c.inv_f = cv.take<float2>(m2);
   c.h_d = cv.take<double>(m2);
+  c.h_f = cv.take<float2>(m2);
   c.scale = cv.take<double>(2);
   c.exhausted = cv.take<int>(1);
   c.out = cv.take<double>(64);
@@ -461,6 +469,7 @@ __global__ void k_init_coefs(Coefs c, int m2) {
     c.inv_d[i] = 0;
     c.inv_f[i] = make_float2(0, 0);
     c.h_d[i] = 0;
+    c.h_f[i] = make_float2(0, 0);
     c.sigma[i] = 0;
     c.ua_d[i] = c.ub_d[i] = c.uc_d[i] = 0;
     c.ua_f[i] = c.ub_f[i] = c.uc_f[i] = make_float2(0, 0);
