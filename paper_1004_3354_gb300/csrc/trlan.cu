@@ -15,8 +15,8 @@
 //   basis vector (which also removes the s_i u_i components of H v_l).
 //
 // The projected eigenproblem (dense, symmetric, at most ED_MAX_BASIS rows) is
-// solved on the device by cyclic Jacobi in one block (round-robin pairs, all
-// disjoint rotations of a round at once); the basis rotation V_m Y is k_ritz.
+// solved on the device by cyclic Jacobi in one block, float sweeps finished in
+// FP64; the basis rotation V_m Y is k_ritz.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -31,113 +31,270 @@ namespace {
 
 constexpr int kMaxBasis = ED_MAX_BASIS;
 constexpr int kJacThreads = 512;
+constexpr int kJacPairs = kMaxBasis / 2;
+
+// Row stride of a matrix of mp rows in shared memory (odd: rows fall into
+// different banks).
+__host__ __device__ inline int jac_ld(int mp) { return mp + 1; }
+// Both the matrix and the vectors in shared memory up to this size; larger
+// bases keep the vectors in global scratch.
+constexpr int kJacSmemRows = 112;
+inline size_t jac_smem(int m) {
+  const int mp = m + (m & 1);
+  const size_t one = (size_t)mp * jac_ld(mp) * sizeof(double);
+  return (mp <= kJacSmemRows ? 2 : 1) * one + (size_t)kJacPairs * (kJacPairs + 1) / 2 * sizeof(uint16_t);
+}
+
+// tangent of the rotation that annihilates a_pq, from d = a_qq - a_pp and a = 2 a_pq
+__device__ __forceinline__ float jac_tan(float d, float a) {
+  const float tau = d / a;
+  return (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+}
+__device__ __forceinline__ void jac_cs(float t, float& c, float& s) {
+  c = rsqrtf(1.f + t * t);
+  s = t * c;
+}
+// cosine and sine of a given tangent to FP64 accuracy: two Newton steps from a
+// float reciprocal root (c^2 + s^2 = 1 is what keeps the vectors orthogonal)
+__device__ __forceinline__ void jac_cs(double t, double& c, double& s) {
+  const double d = fma(t, t, 1.0);
+  double y = (double)rsqrtf((float)d);
+  y = y * fma(-0.5 * d, y * y, 1.5);
+  y = y * fma(-0.5 * d, y * y, 1.5);
+  c = y;
+  s = t * y;
+}
+
+// Rotations of one round, by the first np threads: pair i of round r in the
+// round-robin order, identity where |a_pq| <= skip; inv scales the matrix to
+// entries of about 1 for the float tangent.
+template <class T>
+__device__ __forceinline__ void jac_params(const T* A, int ld, int mp, int r, T skip, T inv, T* cs, T* sn, int* pq) {
+  const int np = mp / 2, i = threadIdx.x;
+  if (i >= np) return;
+  const int a = (i == 0) ? 0 : ((i - 1 + r) % (mp - 1)) + 1;
+  const int b = ((mp - 2 - i + r) % (mp - 1)) + 1;
+  const int p = a < b ? a : b, q = a < b ? b : a;
+  const T apq = A[p * ld + q];
+  T c = T(1), s = T(0);
+  if (fabs(apq) > skip) 
+    jac_cs((T)jac_tan((float)((A[q * ld + q] - A[p * ld + p]) * inv), (float)(2 * apq * inv)), c, s);
+  pq[i] = p << 8 | q;
+  cs[i] = c;
+  sn[i] = s;
+}
+
+// A <- J^T A J over the 2 x 2 blocks of the pairs i <= j (each block depends on
+// its own four entries only, so a round needs no barrier inside), mirrored;
+// Y, which holds the vectors as rows, <- J^T Y.
+template <class T>
+__device__ __forceinline__ void jac_rotate(T* A, T* Y, int ld, int mp, const uint16_t* tab, const T* cs, const T* sn,
+                                           const int* pq) {
+  const int np = mp / 2;
+  for (int idx = threadIdx.x; idx < np * (np + 1) / 2; idx += kJacThreads) {
+    const int i = tab[idx] >> 8, j = tab[idx] & 255;
+    const T si = sn[i], sj = sn[j];
+    if (si == T(0) && sj == T(0)) continue;
+    const T ci = cs[i], cj = cs[j];
+    const int pi = pq[i] >> 8, qi = pq[i] & 255, pj = pq[j] >> 8, qj = pq[j] & 255;
+    const T pp = A[pi * ld + pj], pr = A[pi * ld + qj], qp = A[qi * ld + pj], qr = A[qi * ld + qj];
+    const T a0 = ci * pp - si * qp, b0 = si * pp + ci * qp;   // rows of pair i
+    const T a1 = ci * pr - si * qr, b1 = si * pr + ci * qr;
+    const T r0 = cj * a0 - sj * a1, r1 = sj * a0 + cj * a1;   // columns of pair j
+    const T r2 = cj * b0 - sj * b1, r3 = sj * b0 + cj * b1;
+    A[pi * ld + pj] = r0;
+    A[pi * ld + qj] = r1;
+    A[qi * ld + qj] = r3;
+    if (i == j) {
+      A[qi * ld + pj] = r1;   // the pair's own block stays symmetric
+    } else {
+      A[qi * ld + pj] = r2;
+      A[pj * ld + pi] = r0;
+      A[qj * ld + pi] = r1;
+      A[pj * ld + qi] = r2;
+      A[qj * ld + qi] = r3;
+    }
+  }
+  const int di = kJacThreads / mp, dr = kJacThreads - di * mp;
+  int i = threadIdx.x / mp, r = threadIdx.x - i * mp;
+  while (i < np) {
+    const T s = sn[i];
+    if (s != T(0)) {
+      const T c = cs[i];
+      const int p = pq[i] >> 8, q = pq[i] & 255;
+      const T yp = Y[p * ld + r], yq = Y[q * ld + r];
+      Y[p * ld + r] = c * yp - s * yq;
+      Y[q * ld + r] = s * yp + c * yq;
+    }
+    i += di;
+    r += dr;
+    if (r >= mp) r -= mp, ++i;
+  }
+}
 
 // Eigen-decomposition of the m x m symmetric matrix Ain (row-major, leading
 // dimension lda): theta ascending, eigenvector i in S[i * ldS + r] (and its
-// double-float split in Sf).  Y is m * m doubles of device scratch.
+// double-float split in Sf).  Yg is kMaxBasis^2 doubles of device scratch; S
+// also serves as scratch.
+//
+// Cyclic Jacobi in one block (round-robin pairs, all disjoint rotations of a
+// round at once).  A round of a 40 x 40 matrix is 5,600 FP64 multiply-adds, 2 us
+// at GB300's 1.6 FP64 lanes per SM and clock, and 8 to 10 sweeps of 39 rounds
+// are needed from scratch; in float a round takes 0.2 us.  So the sweeps run in
+// float first, the vectors are made orthonormal in FP64 (two Newton-Schulz
+// steps: Gram matrix in FP64, the small correction's product in float), the
+// matrix is transformed by them in FP64, and FP64 sweeps finish from
+// off-diagonals of about 1e-6 (two sweeps) to the same criterion as sweeps in
+// FP64 throughout.
 __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __restrict__ Ain, int m, int lda,
-                                                            double* __restrict__ theta, double* __restrict__ S,
-                                                            float2* __restrict__ Sf, int ldS, double* __restrict__ Y,
-                                                            int* __restrict__ sweeps) {
-  extern __shared__ double A[];  // m x m, row stride m
-  __shared__ double cs[kMaxBasis / 2], sn[kMaxBasis / 2];
-  __shared__ int pp[kMaxBasis / 2], qq[kMaxBasis / 2];
+                                                            double* __restrict__ theta, double* S,
+                                                            float2* __restrict__ Sf, int ldS, double* Yg) {
+  extern __shared__ __align__(16) unsigned char jsm[];
+  const int mp = m + (m & 1);  // an odd size is padded by a zero row and column (index m)
+  const int ld = jac_ld(mp), np = mp / 2;
+  const size_t one = (size_t)mp * ld;
+  double* A = reinterpret_cast<double*>(jsm);
+  const bool ysm = mp <= kJacSmemRows;
+  double* Y = ysm ? A + one : Yg;
+  uint16_t* tab = reinterpret_cast<uint16_t*>(A + (ysm ? 2 : 1) * one);
+  // float phase: the matrix and its vectors share the FP64 matrix's place
+  float* Af = reinterpret_cast<float*>(A);
+  float* Yf = Af + one;
+  __shared__ double cs[kJacPairs], sn[kJacPairs];
+  __shared__ float csf[kJacPairs], snf[kJacPairs];
+  __shared__ int pq[kJacPairs];
   __shared__ double red[kJacThreads / 32];
   __shared__ int order[kMaxBasis];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < m * m; i += nt) {
-    A[i] = Ain[(size_t)(i / m) * lda + i % m];
-    Y[i] = (i / m == i % m) ? 1.0 : 0.0;
-  }
-  __syncthreads();
+  const int tid = threadIdx.x, nt = kJacThreads;
+  const int lane = tid & 31, warp = tid >> 5, nw = nt / 32;
   auto block_sum = [&](double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
+    if (lane == 0) red[warp] = v;
     __syncthreads();
     double t = 0.0;
-    for (int w = 0; w < nt / 32; ++w) t += red[w];
+    for (int w = 0; w < nw; ++w) t += red[w];
     __syncthreads();
     return t;
   };
-  double fro = 0.0;
-  for (int i = tid; i < m * m; i += nt) fro += A[i] * A[i];
+  auto block_sumf = [&](float v) { return block_sum((double)v); };
+  for (int i = tid; i < kMaxBasis; i += nt) order[i] = i;   // stays valid where values are not comparable (NaN)
+  for (int i = warp; i < np; i += nw)
+    for (int j = lane; j < np; j += 32)
+      if (j >= i) tab[i * np - i * (i - 1) / 2 + (j - i)] = (uint16_t)(i << 8 | j);
+  double fro = 0.0, amax = 0.0;
+  for (int i = warp; i < m; i += nw)
+    for (int j = lane; j < m; j += 32) {
+      const double v = Ain[(size_t)i * lda + j];
+      fro += v * v;
+      amax = fmax(amax, fabs(v));
+    }
   fro = block_sum(fro);
-  const int mp = m + (m & 1);  // players; index m is a dummy when m is odd
-  const int np = mp / 2;
-  int sweep = 0;
-  for (; sweep < 60 && m > 1; ++sweep) {
+  for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if (lane == 0) red[warp] = amax;
+  __syncthreads();
+  for (int w = 0; w < nw; ++w) amax = fmax(amax, red[w]);
+  __syncthreads();
+  // ---- float sweeps on the matrix scaled to entries of at most 1
+  const double inv = amax > 0.0 ? 1.0 / amax : 0.0;
+  for (int i = warp; i < mp; i += nw)
+    for (int j = lane; j < mp; j += 32) {
+      Af[i * ld + j] = (i < m && j < m) ? (float)(Ain[(size_t)i * lda + j] * inv) : 0.f;
+      Yf[i * ld + j] = i == j ? 1.f : 0.f;
+    }
+  __syncthreads();
+  const double frof = fro * inv * inv;
+  for (int sweep = 0; sweep < 12 && m > 1; ++sweep) {
+    float off = 0.f;
+    for (int i = warp; i < m; i += nw)
+      for (int j = lane; j < m; j += 32)
+        if (i != j) off += Af[i * ld + j] * Af[i * ld + j];
+    if (!(block_sumf(off) > 1e-11 * frof)) break;
+    for (int r = 0; r < mp - 1; ++r) {
+      jac_params<float>(Af, ld, mp, r, 0.f, 1.f, csf, snf, pq);
+      __syncthreads();
+      jac_rotate<float>(Af, Yf, ld, mp, tab, csf, snf, pq);
+      __syncthreads();
+    }
+  }
+  // ---- orthonormal vectors in FP64: twice Y += E Y with E = (I - Y Y^T) / 2
+  for (int i = warp; i < mp; i += nw)
+    for (int j = lane; j < mp; j += 32) Y[i * ld + j] = (double)Yf[i * ld + j];
+  __syncthreads();
+  for (int step = 0; step < 2; ++step) {
+    for (int idx = tid; idx < m * m; idx += nt) {
+      const int i = idx / m, j = idx - i * m;
+      if (j > i) continue;
+      double g = 0.0;
+      for (int r = 0; r < m; ++r) g = fma(Y[i * ld + r], Y[j * ld + r], g);
+      const float e = (float)(0.5 * ((i == j ? 1.0 : 0.0) - g));
+      Af[i * ld + j] = e;
+      Af[j * ld + i] = e;
+    }
+    __syncthreads();
+    for (int i = warp; i < m; i += nw)
+      for (int r = lane; r < m; r += 32) {
+        float v = 0.f;
+        for (int j = 0; j < m; ++j) v = fmaf(Af[i * ld + j], Yf[j * ld + r], v);
+        Y[i * ld + r] += (double)v;
+      }
+    __syncthreads();
+  }
+  // ---- B = Y A Y^T through T[r][v] = sum_c A[r][c] Y[v][c] (kept in S); A is
+  // an arrow on a tridiagonal, so most of its entries are zero
+  for (int r = warp; r < m; r += nw)
+    for (int v = lane; v < m; v += 32) {
+      double t = 0.0;
+      for (int c = 0; c < m; ++c) {
+        const double arc = Ain[(size_t)r * lda + c];
+        if (arc != 0.0) t = fma(arc, Y[v * ld + c], t);
+      }
+      S[(size_t)r * ldS + v] = t;
+    }
+  __syncthreads();
+  for (int idx = tid; idx < mp * mp; idx += nt) {
+    const int u = idx / mp, v = idx - u * mp;
+    if (v > u) continue;
+    double t = 0.0;
+    if (u < m)
+      for (int r = 0; r < m; ++r) t = fma(Y[u * ld + r], S[(size_t)r * ldS + v], t);
+    A[u * ld + v] = t;
+    A[v * ld + u] = t;
+  }
+  __syncthreads();
+  // ---- FP64 sweeps
+  const double skip = 1e-18 * sqrt(fro) / (double)m;   // below this a whole matrix of entries is under the criterion
+  for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
     double off = 0.0;
-    for (int i = tid; i < m * m; i += nt)
-      if (i / m != i % m) off += A[i] * A[i];
+    for (int i = warp; i < m; i += nw)
+      for (int j = lane; j < m; j += 32)
+        if (i != j) off += A[i * ld + j] * A[i * ld + j];
     off = block_sum(off);
     if (!(off > 1e-32 * fro)) break;
     for (int r = 0; r < mp - 1; ++r) {
-      for (int i = tid; i < np; i += nt) {
-        const int a = (i == 0) ? 0 : ((i - 1 + r) % (mp - 1)) + 1;
-        const int b = ((mp - 2 - i + r) % (mp - 1)) + 1;
-        const int p = a < b ? a : b, q = a < b ? b : a;
-        double c = 1.0, s = 0.0;
-        if (q < m) {
-          const double apq = A[p * m + q];
-          if (apq != 0.0) {
-            const double tau = (A[q * m + q] - A[p * m + p]) / (2.0 * apq);
-            const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
-          }
-        }
-        pp[i] = p;
-        qq[i] = q;
-        cs[i] = c;
-        sn[i] = s;
-      }
+      jac_params<double>(A, ld, mp, r, skip, inv, cs, sn, pq);
       __syncthreads();
-      // A <- J^T A (rows p, q of each pair)
-      for (int idx = tid; idx < np * m; idx += nt) {
-        const int i = idx / m, col = idx % m, p = pp[i], q = qq[i];
-        if (q >= m) continue;
-        const double c = cs[i], s = sn[i], ap = A[p * m + col], aq = A[q * m + col];
-        A[p * m + col] = c * ap - s * aq;
-        A[q * m + col] = s * ap + c * aq;
-      }
-      __syncthreads();
-      // A <- A J (columns p, q) and the eigenvector matrix (Y holds its columns as rows)
-      for (int idx = tid; idx < np * m; idx += nt) {
-        const int i = idx / m, row = idx % m, p = pp[i], q = qq[i];
-        if (q >= m) continue;
-        const double c = cs[i], s = sn[i];
-        const double ap = A[row * m + p], aq = A[row * m + q];
-        A[row * m + p] = c * ap - s * aq;
-        A[row * m + q] = s * ap + c * aq;
-        const double yp = Y[p * m + row], yq = Y[q * m + row];
-        Y[p * m + row] = c * yp - s * yq;
-        Y[q * m + row] = s * yp + c * yq;
-      }
+      jac_rotate<double>(A, Y, ld, mp, tab, cs, sn, pq);
       __syncthreads();
     }
   }
-  if (tid == 0) {
-    for (int i = 0; i < m; ++i) order[i] = i;
-    for (int i = 1; i < m; ++i) {  // insertion sort by eigenvalue
-      const int v = order[i];
-      const double key = A[v * m + v];
-      int j = i - 1;
-      while (j >= 0 && A[order[j] * m + order[j]] > key) {
-        order[j + 1] = order[j];
-        --j;
-      }
-      order[j + 1] = v;
+  // ---- ascending order: a value's place is the number of values before it
+  for (int i = tid; i < m; i += nt) {
+    const double key = A[i * ld + i];
+    int at = 0;
+    for (int j = 0; j < m; ++j) {
+      const double o = A[j * ld + j];
+      at += (o < key || (o == key && j < i)) ? 1 : 0;
     }
-    if (sweeps) *sweeps = sweep;
+    order[at] = i;
   }
   __syncthreads();
-  for (int i = tid; i < m; i += nt) theta[i] = A[order[i] * m + order[i]];
-  for (int idx = tid; idx < m * m; idx += nt) {
-    const int i = idx / m, r = idx % m;
-    const double v = Y[order[i] * m + r];
-    S[(size_t)i * ldS + r] = v;
-    Sf[(size_t)i * ldS + r] = df_from_double(v);
-  }
+  for (int i = tid; i < m; i += nt) theta[i] = A[order[i] * ld + order[i]];
+  for (int i = warp; i < m; i += nw)
+    for (int r = lane; r < m; r += 32) {
+      const double v = Y[order[i] * ld + r];
+      S[(size_t)i * ldS + r] = v;
+      Sf[(size_t)i * ldS + r] = df_from_double(v);
+    }
 }
 
 // Projected matrix of the current basis (size rows): the kept Ritz values and
@@ -167,12 +324,10 @@ __global__ void k_tr_keep(const double* __restrict__ theta, const double* __rest
 
 int jacobi(cudaStream_t st, const double* Hp, int m, int ld, double* theta, double* S, float2* Sf, int ldS,
            double* Y) {
-  const size_t smem = (size_t)m * m * sizeof(double);
-  // one cap for every size (kMaxBasis^2 doubles): concurrent solves of different
-  // basis sizes set the same value
+  // one cap for every size: concurrent solves of different basis sizes set the same value
   ED_TRY_CUDA(cudaFuncSetAttribute(k_sym_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)((size_t)kMaxBasis * kMaxBasis * sizeof(double))));
-  k_sym_jacobi<<<1, kJacThreads, smem, st>>>(Hp, m, ld, theta, S, Sf, ldS, Y, nullptr);
+                                   (int)jac_smem(kJacSmemRows)));
+  k_sym_jacobi<<<1, kJacThreads, jac_smem(m), st>>>(Hp, m, ld, theta, S, Sf, ldS, Y);
   ED_LAUNCH_CHECK();
   return ED_OK;
 }
@@ -198,7 +353,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   // slots padded to 32 elements, so that each starts 16-byte aligned
   const uint64_t ld = pad32(n);
   ED_TRY(vb.alloc(ctx, ((size_t)m + 2 + n_rot) * ld * eb));
-  ED_TRY(cb.alloc(ctx, coef_bytes(m, 1) + (size_t)kMaxBasis * kMaxBasis * 8 * 4 + (size_t)kMaxBasis * 8 * 8));
+  ED_TRY(cb.alloc(ctx, coef_bytes(m, 1) + (size_t)kMaxBasis * kMaxBasis * 8 * 4 + (size_t)kMaxBasis * 8 * 16));
   ED_TRY(hb.alloc(ctx, cgs_part<V>(ctx, n, m) * sizeof(double)));
   V* Vb = static_cast<V*>(vb.p);
   V* w = Vb + (size_t)(m + 1) * ld;
@@ -207,7 +362,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   Coefs c = carve_coefs(cv, m);
   const int ldS = kMaxBasis;
   double* Hp = cv.take<double>((size_t)kMaxBasis * kMaxBasis);
-  double* Y = cv.take<double>((size_t)kMaxBasis * kMaxBasis);
+  double* Y = cv.take<double>((size_t)kMaxBasis * jac_ld(kMaxBasis));
   double* Sd = cv.take<double>((size_t)kMaxBasis * ldS);
   float2* Sf = cv.take<float2>((size_t)kMaxBasis * ldS);
   double* theta = cv.take<double>(kMaxBasis);

@@ -96,3 +96,28 @@ def test_tridiagonal_solver_scales(env, power):
         assert np.all(np.abs(ev - ref) <= 1e-12 * np.max(np.abs(ref))), ev - ref
     finally:
         ed.ed_sector_destroy(sec)
+
+
+@pytest.mark.parametrize("m_b", [5, 6, 39, 40, 112, 113, 127, 128])
+def test_projected_eigensolver_sizes(env, m_b):
+    """Thick restart with every kind of projected matrix: odd (padded by a zero
+    row) and even, the vectors in shared memory (up to 112 rows) or in global
+    scratch.  Values to 1e-12 ||H|| (FP64 rounding over a few hundred rotations
+    of entries below 30), vectors orthonormal to 1e-12, residuals as the
+    tolerance allows."""
+    ed, ctx, torch = env
+    m = W.aim(8, seed=4)
+    H = osec.build_csr(m, 4, 3)
+    n, k, tol = H.shape[0], 3, 1e-10
+    ref = np.linalg.eigvalsh(H.toarray())
+    scale = np.max(np.abs(ref))
+    sec = ed.ed_sector_create(ctx, m, 4, 3, "fp64")
+    try:
+        v = empty_vec(n, "fp64", ed, torch, count=k)
+        ev, _, _ = ed.ed_lanczos_tr(sec, k=k, tol=tol, max_basis=m_b, max_iter=20000, check_every=5, evecs=v)
+        assert np.all(np.abs(ev - ref[:k]) <= 1e-12 * scale), ev - ref[:k]
+        X = v.cpu().numpy().reshape(k, n)
+        assert np.max(np.abs(X @ X.T - np.eye(k))) <= 1e-12
+        assert np.max(np.linalg.norm(H @ X.T - X.T * ev, axis=0)) <= 2 * tol * max(1.0, scale)
+    finally:
+        ed.ed_sector_destroy(sec)
