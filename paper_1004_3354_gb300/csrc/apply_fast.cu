@@ -246,17 +246,10 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
         ok[e] = d < D;
         dv[e] = ok[e] ? d : d0;
       }
-      C dg[4];
-      ld4<C>(ddr + 4 * (uint64_t)ent, dg);
       const uchar4 c4 = __ldg(F.cnt4 + w);
       A acc[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const V xv = xs[dv[e]];
-        acc[e] = P::zero();
-        P::mac(acc[e], dg[e], xv);
-        P::mac(acc[e], eu, xv);
-      }
+      for (int e = 0; e < 4; ++e) acc[e] = P::zero();
       // down hops: slot counts descend (c0 >= c1 >= c2 >= c3), so the first c3
       // steps serve all four slots, the next c2 - c3 three, and so on
       {
@@ -305,10 +298,9 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
           }
           const C c0 = lcw[k], c1 = lcw[k + 1];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            P::mac(acc[e], c0, a0[e]);
-            P::mac(acc[e], c1, a1[e]);
-          }
+          for (int e = 0; e < 4; ++e) P::mac(acc[e], c0, a0[e]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) P::mac(acc[e], c1, a1[e]);
         }
         if (k < nlw) {
           const V* x0 = x + lrw[k];
@@ -347,6 +339,19 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
               if (mvv >= 0) P::mac(acc[e], (mvv & 1) ? P::neg(cj) : cj, __ldg(xm + (uint32_t)(mvv >> 1)));
             }
           }
+        }
+      }
+      // the diagonal last: it is the largest term, and a double-float sum's
+      // rounding follows the size of its partial sums (a third of the error of
+      // the diagonal first)
+      {
+        C dg[4];
+        ld4<C>(ddr + 4 * (uint64_t)ent, dg);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const V xv = xs[dv[e]];
+          P::mac(acc[e], dg[e], xv);
+          P::mac(acc[e], eu, xv);
         }
       }
 #pragma unroll
@@ -432,8 +437,8 @@ size_t pair_smem(uint32_t D, int n_coef) {
          align16(kList * 8) + align16(kMaxDelta * 4);
 }
 
-// The two rows' multiply-adds of a pair, lane-wise exactly df_mac (XLO, x in
-// double-float) or df_mac1 (float x).  Double-float rows run them as scalar
+// The two rows' multiply-adds of a pair: df_mac on each (XLO, x in
+// double-float) or the paired form (float x).  Double-float rows run them as scalar
 // FP32 instructions (0.70 ms against 0.78 ms with f32x2 at N_s = 15), float
 // rows as f32x2 instructions (0.49 ms against 0.55 ms scalar).
 template <bool XLO>
@@ -570,13 +575,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_pair(FastView F, const typen
       ld4<float2>(ddB + 4 * (uint64_t)ent, dgb);
       float2 H[4], L[4];  // (A, B) hi and lo parts of the four slots
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const PV X = xs[dv[e]];
-        H[e] = L[e] = make_float2(0.f, 0.f);
-        df_mac2s<XLO>(H[e], L[e], make_float2(dga[e].x, dgb[e].x), make_float2(dga[e].y, dgb[e].y), T::hi(X),
-                     T::lo(X));
-        df_mac2s<XLO>(H[e], L[e], EUh, EUl, T::hi(X), T::lo(X));
-      }
+      for (int e = 0; e < 4; ++e) H[e] = L[e] = make_float2(0.f, 0.f);
       // down hops: slot counts descend (c0 >= c1 >= c2 >= c3)
       {
         const uchar4 c4 = __ldg(F.cnt4 + w);
@@ -606,6 +605,14 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_pair(FastView F, const typen
           ED_HOP(0, h.x);
         }
 #undef ED_HOP
+      }
+      // the diagonal between the down and the up hops, as in the one-row kernel
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const PV X = xs[dv[e]];
+        df_mac2s<XLO>(H[e], L[e], make_float2(dga[e].x, dgb[e].x), make_float2(dga[e].y, dgb[e].y), T::hi(X),
+                     T::lo(X));
+        df_mac2s<XLO>(H[e], L[e], EUh, EUl, T::hi(X), T::lo(X));
       }
       // up hops: the k-th neighbour row of A and of B
       for (int k = 0; k < nup; ++k) {

@@ -313,10 +313,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_nat(NatView F, const typenam
       } else {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const C dg = __ldg(F.dd + (uint64_t)pus[r] * NE + d);
           Aa[r] = P::zero();
-          P::mac(Aa[r], dg, xv.v[r]);
-          P::mac(Aa[r], eus[r], xv.v[r]);
           Bb[r] = P::zero();
         }
       }
@@ -397,6 +394,14 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_nat(NatView F, const typenam
           }
 #pragma unroll
           for (int i = 0; i < 2; ++i) h[i] = hn[i];
+        }
+      }
+      if constexpr (!kF32) {   // after the down hops: the largest term last keeps the partial sums' rounding small
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const C dg = __ldg(F.dd + (uint64_t)pus[r] * NE + d);
+          P::mac(Aa[r], dg, xv.v[r]);
+          P::mac(Aa[r], eus[r], xv.v[r]);
         }
       }
       // pass B: CH steps per round trip

@@ -325,32 +325,37 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
 }
 
 // acc (hi, lo) += c (hi, lo) * x (hi, lo); the lo part accumulates lazily.
+// Eleven float instructions.  With p = fl(c.x x.x) and s = fl(acc.x + p),
+// Knuth's TwoSum error of that sum is v + (p - bb), bb = fl(s - acc.x); the
+// product's own error c.x x.x - p joins it in one fused multiply-add, c.x x.x -
+// bb rounded once.  The cross terms c.x x.y + c.y x.x stay a chain of their own:
+// taking them into the error's chain saves one more instruction and is slower
+// (N_s = 15 H*v: 638 us against 572 us; 602 us with separate product and sum
+// errors, twelve instructions).
 __device__ __forceinline__ void df_mac(float2& acc, float2 c, float2 x) {
-  float p = __fmul_rn(c.x, x.x);
-  float e = __fmaf_rn(c.x, x.x, -p);
-  e = __fmaf_rn(c.x, x.y, e);
-  e = __fmaf_rn(c.y, x.x, e);
-  float s, t;
-  two_sum(acc.x, p, s, t);
+  const float s = __fadd_rn(acc.x, __fmul_rn(c.x, x.x));
+  const float nb = __fsub_rn(acc.x, s);                     // -bb
+  const float v = __fsub_rn(acc.x, __fadd_rn(s, nb));
+  const float e = __fmaf_rn(c.x, x.y, __fmul_rn(c.y, x.x));
+  acc.y = __fadd_rn(acc.y, __fadd_rn(e, __fadd_rn(v, __fmaf_rn(c.x, x.x, nb))));
   acc.x = s;
-  acc.y = __fadd_rn(acc.y, __fadd_rn(t, e));
 }
 
 // acc += c * x with x a plain float.
 __device__ __forceinline__ void df_mac1(float2& acc, float2 c, float x) {
-  float p = __fmul_rn(c.x, x);
-  float e = __fmaf_rn(c.x, x, -p);
-  e = __fmaf_rn(c.y, x, e);
-  float s, t;
-  two_sum(acc.x, p, s, t);
+  const float s = __fadd_rn(acc.x, __fmul_rn(c.x, x));
+  const float nb = __fsub_rn(acc.x, s);
+  const float v = __fsub_rn(acc.x, __fadd_rn(s, nb));
+  acc.y = __fadd_rn(acc.y, __fmaf_rn(c.y, x, __fadd_rn(v, __fmaf_rn(c.x, x, nb))));
   acc.x = s;
-  acc.y = __fadd_rn(acc.y, __fadd_rn(t, e));
 }
 
 // Two independent double-float accumulators at once with the paired FP32
 // instructions (add/sub/mul/fma .f32x2): H = (hi0, hi1), L = (lo0, lo1) take
-// (Ch, Cl) * (Xh, Xl) lane-wise, each lane exactly as df_mac (or as df_mac1
-// when XLO is false and x is a plain float).
+// (Ch, Cl) * (Xh, Xl) lane-wise (x a plain float when XLO is false).  The
+// product P is formed on its own, with its error beside the sum's: in df_mac's
+// shorter form P feeds only the sum and gets fused into it, and the sum's error
+// then no longer follows from TwoSum.
 __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
   float2 d;
   asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
