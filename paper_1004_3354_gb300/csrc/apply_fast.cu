@@ -73,18 +73,30 @@ struct FastView {
   int n_lp;                     // term lists per row: 2^M with the delta layout, else 1
   uint32_t lcap;                // capacity of one list: longest up-hop plus spin-flip / pair-hop list
   double* dotp;                 // optional: per-block partial sums of <x, y>
+  // general diagonal (models whose interaction window spans several 8-site
+  // chunks): dd holds e_dn alone, and the cross tables' rows of the up string
+  // are staged per row
+  const uint4* gpat4;           // [n_win*32] window bits of four entries per lane: sd >> w_lo
+  const uint32_t* ub;           // up strings
+  int n_chunks, w_lo;
+  int w_bits[4];
+  uint32_t w_off[4];
+  const double* W;
+  const float2* W_df;
 };
+
+constexpr int kChunkRow = 256;  // entries of one cross table row (8 sites)
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 template <class P>
-size_t fast_smem(uint32_t D, int n_coef, int n_lp, uint32_t lcap) {
+size_t fast_smem(uint32_t D, int n_coef, int n_lp, uint32_t lcap, int n_chunks = 0) {
   using V = typename P::V;
   using C = typename P::C;
   const size_t nl = (size_t)n_lp * lcap;
   return align16(D * sizeof(V)) + align16(n_coef * sizeof(C)) + align16(nl * sizeof(C)) + align16(kList * sizeof(C)) +
          align16(nl * sizeof(int64_t)) + align16(kList * sizeof(uint64_t)) + align16(kList * 4) +
-         align16(kMaxDelta * 4) + align16((size_t)n_lp * 4);
+         align16(kMaxDelta * 4) + align16((size_t)n_lp * 4) + (size_t)n_chunks * kChunkRow * sizeof(C);
 }
 
 // four consecutive table entries (16-byte aligned)
@@ -122,7 +134,9 @@ __device__ __forceinline__ uint32_t sel4(const uint4& v, int e) {
   return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w));
 }
 
-template <class P, int BS, int MINB>
+// GEN: the general diagonal (several cross-table chunks) instead of one table
+// row per up-string pattern.
+template <class P, int BS, int MINB, bool GEN = false>
 __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typename P::V* __restrict__ x,
                                                        typename P::V* __restrict__ y) {
   using V = typename P::V;
@@ -154,6 +168,8 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
   int32_t* mds = reinterpret_cast<int32_t*>(p);   // move shifts per pattern
   p += align16(kMaxDelta * 4);
   int* ln = reinterpret_cast<int*>(p);            // list lengths
+  p += align16((size_t)F.n_lp * 4);
+  C* ws = reinterpret_cast<C*>(p);                // the row's cross-table rows (GEN)
   __shared__ int n_up_s, n_mx_s;
   __shared__ uint32_t pat_s;
   const bool mixd = F.dpat4 != nullptr;
@@ -220,10 +236,18 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
         mm[k] = mixd ? (uint32_t)F.mx_mv[m0 + k] * (uint32_t)F.np : (uint32_t)F.mx_mv[m0 + k] * D;
       }
     }
+    if (GEN) {
+      const uint32_t su = F.ub[u] >> F.w_lo;
+      for (int c = 0; c < F.n_chunks; ++c) {
+        const int nb = 1 << F.w_bits[c];
+        const size_t row = F.w_off[c] + ((size_t)((su >> (8 * c)) & (nb - 1)) << F.w_bits[c]);
+        for (int k = threadIdx.x; k < nb; k += BS) ws[c * kChunkRow + k] = P::ld(F.W, F.W_df, row + k);
+      }
+    }
     if (threadIdx.x == 0) {
       n_up_s = (int)nh;
       n_mx_s = (int)nm;
-      pat_s = F.row_pat[u];
+      pat_s = GEN ? 0u : F.row_pat[u];
     }
     cp_async_wait_all();
     __syncthreads();
@@ -347,11 +371,17 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
       {
         C dg[4];
         ld4<C>(ddr + 4 * (uint64_t)ent, dg);
+        const uint4 gq = GEN ? __ldg(F.gpat4 + ent) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const V xv = xs[dv[e]];
           P::mac(acc[e], dg[e], xv);
           P::mac(acc[e], eu, xv);
+          if (GEN) {
+            const uint32_t pt = sel4(gq, e);
+            for (int c = 0; c < F.n_chunks; ++c)
+              P::mac(acc[e], ws[c * kChunkRow + ((pt >> (8 * c)) & ((1u << F.w_bits[c]) - 1u))], xv);
+          }
         }
       }
 #pragma unroll
@@ -727,7 +757,7 @@ __global__ void k_win_tables(uint32_t D, uint32_t n_win, uint32_t max_cnt, const
                              const double* __restrict__ coef, int n_coef, int zero_id, int vbytes, int cbytes,
                              uint32_t* __restrict__ hop, const double* __restrict__ e_dn,
                              const double* __restrict__ W, int w_lo, int wbits, int n_pat, double* __restrict__ dd,
-                             int orb0, uint8_t* __restrict__ dpat) {
+                             int orb0, uint8_t* __restrict__ dpat, uint32_t* __restrict__ gpat) {
   const uint64_t NE = (uint64_t)n_win * kWin;
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= NE) return;
@@ -757,6 +787,7 @@ __global__ void k_win_tables(uint32_t D, uint32_t n_win, uint32_t max_cnt, const
     dd[(uint64_t)pu * NE + idx] = v;
   }
   if (dpat) dpat[idx] = (uint8_t)(real ? (s >> orb0) : 0u);
+  if (gpat) gpat[idx] = s >> w_lo;
 }
 
 // Rank shift of each impurity move (x -> y) for each pattern p, read off the
@@ -827,15 +858,25 @@ FastView make_view(const Sector* s) {
   F.mx_mv = s->mx_mv;
   F.n_lp = f.n_lp;
   F.lcap = f.lcap;
+  F.gpat4 = reinterpret_cast<const uint4*>(f.gpat);
+  F.ub = s->up.basis;
+  F.n_chunks = f.gen_ok ? s->n_chunks : 0;
+  F.w_lo = s->w_lo;
+  for (int c = 0; c < 4; ++c) {
+    F.w_bits[c] = s->w_bits[c];
+    F.w_off[c] = s->w_off[c];
+  }
+  F.W = s->W;
+  F.W_df = s->W_df;
   return F;
 }
 
-template <class P, int BS, int MINB>
+template <class P, int BS, int MINB, bool GEN = false>
 int launch_fast(const Sector* s, const void* x, void* y, cudaStream_t st, double* dotp, int* nparts) {
   FastView F = make_view<P>(s);
   F.dotp = dotp;
-  size_t smem = fast_smem<P>(F.D, F.n_coef, F.n_lp, F.lcap);
-  auto kern = k_apply_win<P, BS, MINB>;
+  size_t smem = fast_smem<P>(F.D, F.n_coef, F.n_lp, F.lcap, F.n_chunks);
+  auto kern = k_apply_win<P, BS, MINB, GEN>;
   ED_TRY(smem_cap(s->ctx, kern, smem));
   int per_sm = 0;
   ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem));
@@ -897,9 +938,10 @@ int run_variant(const Sector* s, int v, const void* x, void* y, cudaStream_t st,
 }  // namespace
 
 int build_fast(Sector* s) {
-  s->fast.ok = false;
+  s->fast.ok = s->fast.gen_ok = false;
   const uint32_t D = s->dn.D;
-  if (D < 512 || s->n_chunks > 1 || s->up.max_hops > (uint32_t)kList || s->max_mix > (uint32_t)kList)
+  const bool gen = s->n_chunks > 1;   // general diagonal: the one-row kernel only
+  if (D < 512 || s->up.max_hops > (uint32_t)kList || s->max_mix > (uint32_t)kList)
     return ED_OK;
   if (s->dn.max_hops > 255) return ED_OK;
   if (s->dn_move && s->M * s->M > kList) return ED_OK;
@@ -931,12 +973,14 @@ int build_fast(Sector* s) {
   const size_t vbytes = elem_bytes(s->prec);
   if ((uint64_t)D * vbytes >= (1ull << 19)) return ED_OK;
   const int nc = (int)coef.size();
-  const bool mix_delta = s->dn_move && s->orb0 + s->M == s->n_s && s->M * s->M * (1 << s->M) <= kMaxDelta;
+  const bool mix_delta = !gen && s->dn_move && s->orb0 + s->M == s->n_s && s->M * s->M * (1 << s->M) <= kMaxDelta;
   const int n_lp = mix_delta ? 1 << s->M : 1;
   const uint32_t lcap = std::max(1u, s->up.max_hops + (mix_delta ? s->max_mix : 0u));
-  if (std::max(fast_smem<PolF64>(D, nc, n_lp, lcap), fast_smem<PolDF>(D, nc, n_lp, lcap)) > 220 * 1024) return ED_OK;
+  const int n_ch = gen ? s->n_chunks : 0;
+  if (std::max(fast_smem<PolF64>(D, nc, n_lp, lcap, n_ch), fast_smem<PolDF>(D, nc, n_lp, lcap, n_ch)) > 220 * 1024)
+    return ED_OK;
   const size_t smem2 = s->prec == ED_PREC_DF64 ? pair_smem<PolDF>(D, nc) : pair_smem<PolF32>(D, nc);
-  const bool pair = s->prec != ED_PREC_FP64 && (uint64_t)D * 2 * vbytes < (1ull << 19) && smem2 <= 220 * 1024;
+  const bool pair = !gen && s->prec != ED_PREC_FP64 && (uint64_t)D * 2 * vbytes < (1ull << 19) && smem2 <= 220 * 1024;
 
   // window-local order: inside each window of 128 ranks, longest hop list first
   const uint32_t n_win = (D + kWin - 1) / kWin;
@@ -1022,6 +1066,7 @@ int build_fast(Sector* s) {
   ED_TRY_CUDA(cudaMemcpy(f.row_order, rorder.data(), sizeof(uint32_t) * Du, cudaMemcpyHostToDevice));
   f.mix_delta = mix_delta;
   f.pair_ok = pair;
+  if (gen) ED_TRY(sector_alloc(s, &f.gpat, NE));
   if (mix_delta) {
     const int M = s->M, NP = 1 << M;
     std::vector<uint32_t> dbas(D), wpat(n_win, 0xffffffffu);
@@ -1043,13 +1088,13 @@ int build_fast(Sector* s) {
                                                       s->dn.hop_tgt, s->dn.hop_val, f.coef, f.n_coef, zero_id,
                                                       (int)vbytes, 8,
                                                       f.hop, s->dn.e, (s->n_chunks == 1) ? s->W : nullptr, s->w_lo,
-                                                      wbits, f.n_pat, f.dd, s->orb0, f.dpat);
+                                                      wbits, f.n_pat, f.dd, s->orb0, f.dpat, f.gpat);
   if (pair) {
     ED_TRY(sector_alloc(s, &f.hop2, (size_t)f.max_cnt * NE));
     k_win_tables<<<(unsigned)((NE + 127) / 128), 128>>>(D, n_win, f.max_cnt, f.perm, s->dn.basis, s->dn.hop_ptr,
                                                         s->dn.hop_tgt, s->dn.hop_val, f.coef, f.n_coef, zero_id,
                                                         (int)(2 * vbytes), 16, f.hop2, s->dn.e, nullptr, s->w_lo,
-                                                        wbits, 0, nullptr, s->orb0, nullptr);
+                                                        wbits, 0, nullptr, s->orb0, nullptr, nullptr);
   }
   ED_LAUNCH_CHECK();
   k_row_pat<<<(Du + 127) / 128, 128>>>(Du, s->up.basis, s->w_lo, wbits, f.row_pat);
@@ -1062,6 +1107,10 @@ int build_fast(Sector* s) {
     ED_LAUNCH_CHECK();
   }
   ED_TRY_CUDA(cudaStreamSynchronize(0));  // legacy stream only: leaves other work running
+  if (gen) {
+    f.gen_ok = true;
+    return ED_OK;
+  }
   f.ok = true;
   ED_TRY(build_nat(s, coef, zero_id));
   tune_apply_cached(s);  // a variant tuned earlier for this shape (any creator: ABI, server, Green's function)
@@ -1144,7 +1193,27 @@ int apply_fast_variant(const Sector* s, int v, const void* x, void* y, cudaStrea
   ED_INVALID("unknown precision");
 }
 
+namespace {
+// General diagonal: one row per block, 256 threads x 3 blocks per SM while
+// three staged rows fit, else 384 x 2 (the untuned rule of the one-row kernel).
+template <class P>
+int apply_gen(const Sector* s, const void* x, void* y, cudaStream_t st, double* dotp, int* nparts) {
+  const size_t smem = fast_smem<P>(s->dn.D, s->fast.n_coef, s->fast.n_lp, s->fast.lcap, s->n_chunks);
+  const size_t per_sm = s->ctx->smem_per_sm ? s->ctx->smem_per_sm : 228 * 1024;
+  if (3 * (smem + 1024) <= per_sm) return launch_fast<P, 256, 3, true>(s, x, y, st, dotp, nparts);
+  return launch_fast<P, 384, 2, true>(s, x, y, st, dotp, nparts);
+}
+}  // namespace
+
 int apply_fast(const Sector* s, const void* x, void* y, cudaStream_t st, double* dotp, int* nparts) {
+  if (s->fast.gen_ok) {
+    switch (s->prec) {
+      case ED_PREC_FP64: return apply_gen<PolF64>(s, x, y, st, dotp, nparts);
+      case ED_PREC_DF64: return apply_gen<PolDF>(s, x, y, st, dotp, nparts);
+      case ED_PREC_FP32: return apply_gen<PolF32>(s, x, y, st, dotp, nparts);
+    }
+    ED_INVALID("unknown precision");
+  }
   const int v = fast_variant_applies(s, s->tune) ? s->tune : fast_default_variant(s);
   return apply_fast_variant(s, v, x, y, st, dotp, nparts);
 }

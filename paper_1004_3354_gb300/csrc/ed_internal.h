@@ -184,6 +184,11 @@ struct Sector {
     // ranks; inside a window they are sorted by hop count (longest first) and
     // dealt to 32 lanes x 4 slots, entry index w*128 + lane*4 + slot.
     bool ok = false;
+    // models whose interaction window spans several 8-site chunks (a Hubbard
+    // cluster of more than eight sites): the one-row kernel with the general
+    // diagonal; such a sector has nothing to tune
+    bool gen_ok = false;
+    uint32_t* gpat = nullptr;   // [n_win*128] window bits of each entry (gen_ok)
     uint32_t n_win = 0;         // ceil(D_dn / 128)
     uint32_t max_cnt = 0;       // widest down-hop list
     int n_coef = 0;             // distinct down-hop matrix elements (<= 256), one of them 0.0
@@ -249,6 +254,9 @@ int sector_alloc(Sector* s, T** p, size_t n) {
   }
   return st;
 }
+
+// Whether H*v runs a row kernel of apply_fast.cu (which can also form <x, Hx>).
+inline bool has_rows(const Sector* s) { return s->fast.ok || s->fast.gen_ok; }
 
 // Builders (basis.cu, csr.cu)
 int validate_model(const ed_model* m);

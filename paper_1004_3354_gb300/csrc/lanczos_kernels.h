@@ -370,7 +370,7 @@ size_t cgs_part(const Ctx* c, uint64_t n, int mmax) {
 // H v_j with the partials of <v_j, H v_j> in W.partial; *np of them.
 template <class V>
 int apply_dot(const Sector* s, Work<V>& W, const V* x, V* y, int* np) {
-  if (s->fast.ok) return apply_fast(s, x, y, W.st, W.partial, np);
+  if (has_rows(s)) return apply_fast(s, x, y, W.st, W.partial, np);
   ED_TRY(apply_h(s, x, y, W.st));
   k_dot<V><<<W.grid, kRedThreads, 0, W.st>>>(x, y, W.n, W.partial);
   ED_LAUNCH_CHECK();

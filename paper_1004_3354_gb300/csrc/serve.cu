@@ -88,7 +88,7 @@ struct Run3 {
   V* q(int j) { return Q[((j % 3) + 3) % 3]; }
 
   int apply_dot_launch(const V* x, V* y) {
-    if (s->fast.ok) return apply_fast(s, x, y, st, partial, &np_apply);
+    if (has_rows(s)) return apply_fast(s, x, y, st, partial, &np_apply);
     ED_TRY(apply_h(s, x, y, st));
     k_dot<V><<<sgrid, kRedThreads, 0, st>>>(x, y, n, partial);
     ED_LAUNCH_CHECK();
