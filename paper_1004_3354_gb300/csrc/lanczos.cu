@@ -30,37 +30,42 @@ size_t elem_bytes(int prec) {
 
 namespace {
 // Three-vector recurrence on unnormalised vectors (v_j = sigma_j q_j), two
-// large kernels per step: H q_j fused with <q_j, H q_j>, then the update fused
-// with |q_{j+1}|^2.  The coefficients stay on the device.
+// kernels per step: H q_j fused with <q_j, H q_j>, then the update fused with
+// |q_{j+1}|^2.  The coefficients stay on the device.
 template <class V>
 struct Rec3 {
   Sector* s;
   Work<V>* W;
   V* Q[3];  // q_{j-1}, q_j, q_{j+1} rotate through these
   V* Y;     // H q_j
-  uint32_t sgrid;
+  double thr;
   V* q(int j) { return Q[((j % 3) + 3) % 3]; }
+  uint32_t grid() const { return lz_grid(W->ctx, W->n); }
+  NormPart norms() const { return lz_norm_part(W->partial); }
 
   int init() {  // q_0 already in Q[0]
     return dot_to(*W, (const V*)q(0), (const V*)q(0), OP_SIGMA0, 0);
   }
-  int step(int j, double thr, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr) {
+  int step(int j, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr) {
     int np = 0;
     if (e0) ED_TRY_CUDA(cudaEventRecord(e0, W->st));
     ED_TRY(apply_dot<V>(s, *W, q(j), Y, &np));
     if (e1) ED_TRY_CUDA(cudaEventRecord(e1, W->st));
-    k_finish<<<1, kRedThreads, 0, W->st>>>(W->partial, np, OP_ALPHA_Q, j, W->c, 0.0);
-    k_lz_step<V><<<sgrid, kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,
-                                                   W->partial);
-    k_finish<<<1, kRedThreads, 0, W->st>>>(W->partial, (int)sgrid, OP_BETA_Q, j + 1, W->c, thr);
+    k_lz_step<V><<<grid(), kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,
+                                                   W->partial, np, norms(), thr);
+    ED_LAUNCH_CHECK();
+    return ED_OK;
+  }
+  // beta_m of the last step, ahead of reading the coefficients.
+  int close(int m) {
+    k_lz_close<<<1, 32, 0, W->st>>>(norms(), (int)grid(), W->c, m, thr);
     ED_LAUNCH_CHECK();
     return ED_OK;
   }
   // Regenerate q_{j+1} from q_j, q_{j-1} with the stored coefficients.
   int regen(int j) {
     ED_TRY(apply_h(s, q(j), Y, W->st));
-    k_lz_step<V><<<sgrid, kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,
-                                                   nullptr);
+    k_lz_regen<V><<<grid(), kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j);
     ED_LAUNCH_CHECK();
     return ED_OK;
   }
@@ -73,7 +78,8 @@ int coeffs_impl(Sector* s, const void* phi, int depth, double* n2, double* a, do
   const uint64_t n = s->dim;
   size_t eb = sizeof(V);
   DevBuf vb, cb;
-  ED_TRY(vb.alloc(ctx, 4 * n * eb));
+  const uint64_t ld = pad32(n);   // every vector starts 16-byte aligned
+  ED_TRY(vb.alloc(ctx, 4 * ld * eb));
   ED_TRY(cb.alloc(ctx, coef_bytes(depth, 1)));
   V* vecs = static_cast<V*>(vb.p);
   Carve cv{static_cast<char*>(cb.p)};
@@ -86,12 +92,12 @@ int coeffs_impl(Sector* s, const void* phi, int depth, double* n2, double* a, do
   if (W.grid == 0) W.grid = 1;
   W.partial = ctx->d_red;
   W.c = c;
-  Rec3<V> R{s, &W, {vecs, vecs + n, vecs + 2 * n}, vecs + 3 * n, W.grid};
+  Rec3<V> R{s, &W, {vecs, vecs + ld, vecs + 2 * ld}, vecs + 3 * ld, 1e-12};
   k_init_coefs<<<1, 256, 0, st>>>(c, depth + 2);
   ED_TRY_CUDA(cudaMemcpyAsync(R.q(0), phi, n * eb, cudaMemcpyDeviceToDevice, st));
   ED_TRY(R.init());
-  const double thr = 1e-12;
-  for (int j = 0; j < depth; ++j) ED_TRY(R.step(j, thr));
+  for (int j = 0; j < depth; ++j) ED_TRY(R.step(j));
+  ED_TRY(R.close(depth));
   std::vector<double> hb(depth + 1), ha(depth);
   double norm = 0.0;
   int ex = -1;
@@ -127,7 +133,8 @@ int lanczos3_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evec
   const int kk = std::min<int>(k, (int)n);
   size_t eb = sizeof(V);
   DevBuf vb, cb, v0b;
-  ED_TRY(vb.alloc(ctx, 4 * n * eb));
+  const uint64_t ld = pad32(n);   // every vector starts 16-byte aligned
+  ED_TRY(vb.alloc(ctx, 4 * ld * eb));
   ED_TRY(v0b.alloc(ctx, n * eb));
   ED_TRY(cb.alloc(ctx, coef_bytes(mmax, std::max(kk, 1))));
   V* vecs = static_cast<V*>(vb.p);
@@ -151,7 +158,7 @@ int lanczos3_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evec
   W.c = c;
   uint32_t vgrid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 16);
   if (vgrid == 0) vgrid = 1;
-  Rec3<V> R{s, &W, {vecs, vecs + n, vecs + 2 * n}, vecs + 3 * n, W.grid};
+  Rec3<V> R{s, &W, {vecs, vecs + ld, vecs + 2 * ld}, vecs + 3 * ld, 1e-13};
   k_init_coefs<<<1, 256, 0, st>>>(c, mmax + 2);
   if (o->v0) {
     ED_TRY_CUDA(cudaMemcpyAsync(R.q(0), o->v0, n * eb, cudaMemcpyDeviceToDevice, st));
@@ -162,7 +169,6 @@ int lanczos3_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evec
   ED_TRY(R.init());
   std::vector<double> h_theta(ED_MAX_K), h_res(ED_MAX_K);
   int m = 0, n_conv = 0, status = ED_OK;
-  const double thr = 1e-13;
   // one event pair per step times the H*v launches of the recurrence
   std::vector<cudaEvent_t> evs(2 * (size_t)mmax);
   for (auto& e : evs) ED_TRY_CUDA(cudaEventCreate(&e));
@@ -174,11 +180,12 @@ int lanczos3_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evec
   } evguard{&evs};
   int n_steps = 0;
   for (int j = 0; j < mmax; ++j) {
-    ED_TRY(R.step(j, thr, evs[2 * j], evs[2 * j + 1]));
+    ED_TRY(R.step(j, evs[2 * j], evs[2 * j + 1]));
     n_steps = j + 1;
     m = j + 1;
     bool check = ((m % check_every) == 0) || (m == mmax) || (n <= 4096);
     if (!check) continue;
+    ED_TRY(R.close(m));
     int ex = -1;
     ED_TRY_CUDA(cudaMemcpyAsync(ctx->h_red, c.exhausted, sizeof(int), cudaMemcpyDeviceToHost, st));
     ED_TRY_CUDA(cudaStreamSynchronize(st));
@@ -219,8 +226,7 @@ int lanczos3_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evec
     ED_TRY_CUDA(cudaMemsetAsync(out, 0, (size_t)kc * n * eb, st));
     ED_TRY_CUDA(cudaMemcpyAsync(R.q(0), v0b.p, n * eb, cudaMemcpyDeviceToDevice, st));
     for (int jj = 0; jj < m; ++jj) {
-      for (int i0 = 0; i0 < kc; i0 += 8)
-        k_ritz<V, 8><<<vgrid, 256, 0, st>>>(R.q(jj), n, 1, Sq + jj, Sqf + jj, ldS, i0, std::min(8, kc - i0), out, n, 1);
+      ED_TRY(ritz(ctx, st, (const V*)R.q(jj), n, 1, Sq + jj, Sqf + jj, ldS, kc, out, n, 1));
       if (jj + 1 == m) break;
       ED_TRY(R.regen(jj));
     }
@@ -266,7 +272,7 @@ int dot_async(Ctx* c, const void* x, const void* y, uint64_t n, int prec, double
       break;
     default: ED_INVALID("unknown precision %d", prec);
   }
-  k_finish<<<1, kRedThreads, 0, st>>>(c->d_red, (int)grid, OP_SUM, 0, cf, 0.0);
+  k_finish<<<1, kRedThreads, 0, st>>>(c->d_red, (int)grid, OP_SUM, 0, cf);
   ED_LAUNCH_CHECK();
   return ED_OK;
 }

@@ -57,18 +57,17 @@ struct Coefs {
   int* step;        // device step index for graph-replayed steps (slot < 0 / j < 0 read it)
 };
 
-enum FinishOp { OP_SUM, OP_NEGH, OP_NORM_INV, OP_SIGMA0, OP_ALPHA_Q, OP_BETA_Q };
+enum FinishOp { OP_SUM, OP_NEGH, OP_NORM_INV, OP_SIGMA0 };
 
 // Sum nb partials (one output per block of this kernel) and apply `op`.
 __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict__ partial, int nb, int op,
-                                                        int slot, Coefs c, double thr) {
+                                                        int slot, Coefs c) {
   __shared__ double sh[32];
   int o = blockIdx.x;
   double v = 0.0;
   for (int i = threadIdx.x; i < nb; i += blockDim.x) v += partial[(uint64_t)o * nb + i];
   v = block_reduce(v, sh);
   if (threadIdx.x != 0) return;
-  if (slot < 0) slot = *c.step + (-slot - 1);  // -1: current step j, -2: j + 1
   switch (op) {
     case OP_SUM: c.out[slot + o] = v; break;
     case OP_NEGH:
@@ -90,61 +89,150 @@ __global__ void __launch_bounds__(kRedThreads) k_finish(const double* __restrict
       c.beta[0] = 0.0;
       break;
     }
-    case OP_ALPHA_Q: {  // v = <q_j, H q_j>; alpha_j = sigma_j^2 v
-      const int j = slot;
-      const double sg = c.sigma[j];
-      const double a = sg * sg * v;
+  }
+}
+
+// ------------------------------------------------ vector updates
+// q_out = ua y + ub q_j + uc q_{j-1} element by element in sixteen-byte
+// vectors (every buffer 16-byte aligned); q_out may be the buffer of q_{j-1}.
+// Returns the thread's share of <q_out, q_out> (NORM).
+template <class V, bool NORM, class A>
+__device__ __forceinline__ A lz_combine(const V* __restrict__ y, const V* __restrict__ qj, const V* qjm, V* qout,
+                                        uint64_t n, A ua, A ub, A uc) {
+  using W16 = Vec16<V>;
+  using VT = typename W16::T;
+  constexpr int N = W16::N;
+  A nacc{};
+  const uint64_t nv = n / N;
+  const uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (uint64_t)gridDim.x * blockDim.x;
+  auto one = [&](V yv, V q1, V q0) {
+    A a{};
+    hmac(a, ua, yv);
+    hmac(a, ub, q1);
+    if (qjm) hmac(a, uc, q0);
+    const V q = store_v(a, qout);
+    if (NORM) dmac(nacc, q, q);
+    return q;
+  };
+  for (uint64_t t = g0; t < nv; t += gs) {
+    const VT yv = reinterpret_cast<const VT*>(y)[t], v1 = reinterpret_cast<const VT*>(qj)[t];
+    const VT v0 = qjm ? reinterpret_cast<const VT*>(qjm)[t] : VT{};
+    VT o{};
+#pragma unroll
+    for (int i = 0; i < N; ++i) W16::set(o, i, one(W16::get(yv, i), W16::get(v1, i), W16::get(v0, i)));
+    reinterpret_cast<VT*>(qout)[t] = o;
+  }
+  for (uint64_t i = nv * N + g0; i < n; i += gs) qout[i] = one(y[i], qj[i], qjm ? qjm[i] : V{});
+  return nacc;
+}
+
+// beta_j and sigma_j = 1 / beta_j from v = |q_j|^2, sc the running scale.
+__device__ __forceinline__ void lz_beta(double v, double& sc, double thr, double& beta, double& sigma, bool& dead) {
+  const double b = sqrt(fmax(v, 0.0));
+  sc = fmax(sc, b);
+  dead = !(b > thr * fmax(sc, 1.0));
+  beta = dead ? 0.0 : b;
+  sigma = dead ? 0.0 : 1.0 / b;
+}
+
+// One three-vector step after H q_j (in y): alpha_j from the na partials of
+// <q_j, H q_j>, beta_j from the previous step's nn partials of |q_j|^2
+// (npart[(j - 1) & 1]), then q_{j+1} and the partials of its norm
+// (npart[j & 1]).  Every block forms the step's numbers itself, one warp per
+// sum and one thread for the rest, so a step is two launches (H*v and this)
+// where separate finishing launches made it four; block 0 keeps them.  j < 0:
+// the step index in c.step (graph replays).
+struct NormPart {
+  double* p[2];
+};
+template <class V>
+__global__ void __launch_bounds__(kRedThreads) k_lz_step(const V* __restrict__ y, const V* __restrict__ qj,
+                                                         const V* qjm, V* qout, uint64_t n, Coefs c, int j,
+                                                         const double* __restrict__ apart, int na, NormPart npart,
+                                                         double thr) {
+  using A = typename AccOf<V>::T;
+  __shared__ A sh[32];
+  __shared__ double tot[2];
+  __shared__ A u[3];
+  if (j < 0) j = *c.step;
+  if (j == 0) qjm = nullptr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < 2) {
+    const double* p = warp == 0 ? apart : npart.p[(j + 1) & 1];
+    const int nb = warp == 0 ? na : (j > 0 ? (int)gridDim.x : 0);
+    double v = 0.0;
+    for (int i = lane; i < nb; i += 32) v += p[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) tot[warp] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sc = c.scale[j & 1], beta = 0.0, sg = c.sigma[0];
+    bool dead = false;
+    if (j > 0) lz_beta(tot[1], sc, thr, beta, sg, dead);
+    const double a = sg * sg * tot[0];
+    const double ua = sg, ub = -a * sg, uc = j > 0 ? -beta * c.sigma[j - 1] : 0.0;
+    h_split(u[0], ua);
+    h_split(u[1], ub);
+    h_split(u[2], uc);
+    if (blockIdx.x == 0) {
+      if (j > 0) {
+        c.beta[j] = beta;
+        c.sigma[j] = sg;
+        if (dead && *c.exhausted < 0) *c.exhausted = j;
+      }
       c.alpha[j] = a;
-      *c.scale = fmax(*c.scale, fabs(a));
-      const double ua = sg, ub = -a * sg, uc = (j > 0) ? -c.beta[j] * c.sigma[j - 1] : 0.0;
+      c.scale[(j + 1) & 1] = fmax(sc, fabs(a));
       c.ua_d[j] = ua;
       c.ua_f[j] = df_from_double(ua);
       c.ub_d[j] = ub;
       c.ub_f[j] = df_from_double(ub);
       c.uc_d[j] = uc;
       c.uc_f[j] = df_from_double(uc);
-      break;
-    }
-    case OP_BETA_Q: {  // v = |q_{j+1}|^2
-      double b = sqrt(fmax(v, 0.0));
-      double sc = fmax(*c.scale, b);
-      *c.scale = sc;
-      bool dead = !(b > thr * fmax(sc, 1.0));
-      if (dead && *c.exhausted < 0) *c.exhausted = slot;
-      c.beta[slot] = dead ? 0.0 : b;
-      c.sigma[slot] = dead ? 0.0 : 1.0 / b;
-      break;
     }
   }
+  __syncthreads();
+  A nacc = lz_combine<V, true, A>(y, qj, qjm, qout, n, u[0], u[1], u[2]);
+  nacc = block_reduce(nacc, sh);
+  if (threadIdx.x == 0) npart.p[j & 1][blockIdx.x] = to_d(nacc);
 }
 
-// ------------------------------------------------ vector updates
-// q_out = ua_j y + ub_j q_j + uc_j q_{j-1} with block partials of |q_out|^2.
-// q_out may be the buffer of q_{j-1} (element-wise in place).
-template <class V>
-__global__ void __launch_bounds__(kRedThreads) k_lz_step(const V* __restrict__ y, const V* __restrict__ qj,
-                                                         const V* qjm, V* qout, uint64_t n, Coefs c, int j,
-                                                         double* __restrict__ partial) {
-  using A = typename AccOf<V>::T;
-  __shared__ A sh[32];
-  A nacc{};
-  if (j < 0) j = *c.step;
-  if (j == 0) qjm = nullptr;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    typename AccOf<V>::T a{};
-    amac(a, c.ua_d, c.ua_f, j, y[i]);
-    amac(a, c.ub_d, c.ub_f, j, qj[i]);
-    if (qjm) amac(a, c.uc_d, c.uc_f, j, qjm[i]);
-    const V q = store_v(a, qout);
-    qout[i] = q;
-    if (partial) dmac(nacc, q, q);
-  }
-  if (partial) {
-    nacc = block_reduce(nacc, sh);
-    if (threadIdx.x == 0) partial[blockIdx.x] = to_d(nacc);
-  }
+// beta_m, sigma_m and the exhaustion flag after m steps (m < 0: c.step), ahead of
+// a convergence check; the next step forms the same numbers again.  One warp.
+__global__ void k_lz_close(NormPart npart, int nn, Coefs c, int m, double thr) {
+  if (m < 0) m = *c.step;
+  if (m < 1) return;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nn; i += 32) v += npart.p[(m + 1) & 1][i];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (threadIdx.x != 0) return;
+  double sc = c.scale[m & 1], beta, sg;
+  bool dead;
+  lz_beta(v, sc, thr, beta, sg, dead);
+  c.beta[m] = beta;
+  c.sigma[m] = sg;
+  if (dead && *c.exhausted < 0) *c.exhausted = m;
 }
+
+// q_{j+1} again from y = H q_j and the stored coefficients of step j.
+template <class V>
+__global__ void __launch_bounds__(kRedThreads) k_lz_regen(const V* __restrict__ y, const V* __restrict__ qj,
+                                                          const V* qjm, V* qout, uint64_t n, Coefs c, int j) {
+  using A = typename AccOf<V>::T;
+  A ua, ub, uc;
+  h_pick(ua, c.ua_d, c.ua_f, j);
+  h_pick(ub, c.ub_d, c.ub_f, j);
+  h_pick(uc, c.uc_d, c.uc_f, j);
+  lz_combine<V, false, A>(y, qj, qjm, qout, n, ua, ub, uc);
+}
+
+// Blocks of the three-vector kernels; their norm partials take two such rows.
+inline uint32_t lz_grid(const Ctx* c, uint64_t n) {
+  const uint64_t g = (n + 2 * kRedThreads - 1) / (2 * kRedThreads), most = (uint64_t)c->num_sms * 4;
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({g, most, 1024}));
+}
+// Norm partials in a context's reduction scratch, past the dot products' share.
+inline NormPart lz_norm_part(double* red) { return NormPart{{red + 4096, red + 5120}}; }
 
 // Sq[i*ldS + j] = S[i*ldS + j] * sigma[j] (Ritz coefficients on unnormalised q_j)
 __global__ void k_scale_ritz(const double* __restrict__ S, const double* __restrict__ sigma, int m, int k, int ldS,
@@ -254,27 +342,114 @@ __global__ void k_random(V* __restrict__ v, uint64_t n, uint64_t seed) {
   }
 }
 
-// out_i += sum_{j<m} S[i*ldS + j] V_j   for eigenvectors i in [i0, i0 + kn)
+// out_i (+)= sum_{j<m} S[i*ldS + j] V_j for the eigenvectors i in [i0, i0 + KB),
+// i < k: sixteen bytes of each V_j per thread (slots 16-byte aligned), eight in
+// flight, the coefficients of 32 vectors at a time in shared memory.  av: every
+// output row starts 16-byte aligned, else outputs go element by element.
+// (One element per thread and load: 660 us for eight of 22 vectors of the
+// N_s = 13 sector from a basis of 40, 1.4 TB/s.)
+constexpr int kRitzChunk = 32;
 template <class V, int KB>
-__global__ void k_ritz(const V* __restrict__ Vb, uint64_t stride, int m, const double* __restrict__ Sd,
-                       const float2* __restrict__ Sf, int ldS, int i0, int kn, V* __restrict__ out,
-                       uint64_t n, int accumulate) {
+__global__ void __launch_bounds__(256) k_ritz(const V* __restrict__ Vb, uint64_t stride, int m,
+                                              const double* __restrict__ Sd, const float2* __restrict__ Sf, int ldS,
+                                              int i0, int k, V* out, uint64_t n, int accumulate, int av) {
   using A = typename AccOf<V>::T;
-  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (uint64_t)gridDim.x * blockDim.x) {
-    A acc[KB];
+  using W16 = Vec16<V>;
+  using VT = typename W16::T;
+  constexpr int N = W16::N;
+  __shared__ A cs[kRitzChunk][KB];
+  const int kn = min(KB, k - i0);
+  const uint64_t nv = (n + N - 1) / N, gs = (uint64_t)gridDim.x * 256;
+  const uint64_t rounds = (nv + gs - 1) / gs;   // the same for every thread: barriers inside
+  for (uint64_t r = 0; r < rounds; ++r) {
+    const uint64_t t = r * gs + (uint64_t)blockIdx.x * 256 + threadIdx.x;
+    const bool on = t < nv;
+    const bool whole = on && (t + 1) * N <= n;
+    A acc[KB][N];
 #pragma unroll
-    for (int q = 0; q < KB; ++q) acc[q] = (accumulate && q < kn) ? acc_of(out[(uint64_t)(i0 + q) * n + e]) : A{};
-    for (int j = 0; j < m; ++j) {
-      V vj = Vb[(uint64_t)j * stride + e];
+    for (int q = 0; q < KB; ++q) {
+#pragma unroll
+      for (int c = 0; c < N; ++c) acc[q][c] = A{};
+      if (accumulate && q < kn && on) {
+        const V* o = out + (uint64_t)(i0 + q) * n + t * N;
+        if (av && whole) {
+          const VT v = *reinterpret_cast<const VT*>(o);
+#pragma unroll
+          for (int c = 0; c < N; ++c) acc[q][c] = acc_of(W16::get(v, c));
+        } else {
+#pragma unroll
+          for (int c = 0; c < N; ++c)
+            if (t * N + c < n) acc[q][c] = acc_of(o[c]);
+        }
+      }
+    }
+    for (int j0 = 0; j0 < m; j0 += kRitzChunk) {
+      const int jn = min(kRitzChunk, m - j0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < jn * KB; i += 256) {
+        const int j = i / KB, q = i % KB;
+        A h{};
+        if (q < kn) h_pick(h, Sd, Sf, (size_t)(i0 + q) * ldS + j0 + j);
+        cs[j][q] = h;
+      }
+      __syncthreads();
+      if (on) {
+        const V* vb = Vb + (uint64_t)j0 * stride;
+#pragma unroll 8
+        for (int j = 0; j < jn; ++j) {
+          VT v;
+          if (whole) v = __ldg(reinterpret_cast<const VT*>(vb + (uint64_t)j * stride) + t);
+          else v = tile_ld<V>(vb + (uint64_t)j * stride + t * N, 0, (uint32_t)(n - t * N));
+#pragma unroll
+          for (int q = 0; q < KB; ++q)
+#pragma unroll
+            for (int c = 0; c < N; ++c) hmac(acc[q][c], cs[j][q], W16::get(v, c));
+        }
+      }
+    }
+    if (on) {
 #pragma unroll
       for (int q = 0; q < KB; ++q)
-        if (q < kn) amac(acc[q], Sd, Sf, (i0 + q) * ldS + j, vj);
-    }
+        if (q < kn) {
+          V* o = out + (uint64_t)(i0 + q) * n + t * N;
+          if (av && whole) {
+            VT v{};
 #pragma unroll
-    for (int q = 0; q < KB; ++q)
-      if (q < kn) out[(uint64_t)(i0 + q) * n + e] = store_v(acc[q], out);
+            for (int c = 0; c < N; ++c) W16::set(v, c, store_v(acc[q][c], out));
+            *reinterpret_cast<VT*>(o) = v;
+          } else {
+#pragma unroll
+            for (int c = 0; c < N; ++c)
+              if (t * N + c < n) o[c] = store_v(acc[q][c], out);
+          }
+        }
+    }
   }
+}
+
+// k_ritz over all k outputs, eight, two or one at a time (two double-float or
+// FP64 elements of eight outputs fill the registers; a single output should not
+// pay for eight).
+template <class V>
+int ritz(const Ctx* ctx, cudaStream_t st, const V* Vb, uint64_t stride, int m, const double* Sd, const float2* Sf, int ldS,
+         int k, V* out, uint64_t n, int accumulate) {
+  const uint64_t nv = (n + Vec16<V>::N - 1) / Vec16<V>::N;
+  const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((nv + 255) / 256, (uint64_t)ctx->num_sms * 8));
+  const int av = (n * sizeof(V)) % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+  for (int i0 = 0; i0 < k;) {
+    if (k - i0 >= 3) {
+      k_ritz<V, 8><<<grid, 256, 0, st>>>(Vb, stride, m, Sd, Sf, ldS, i0, k, out, n, accumulate, av);
+      i0 += 8;
+    } else if (k - i0 == 2) {
+      k_ritz<V, 2><<<grid, 256, 0, st>>>(Vb, stride, m, Sd, Sf, ldS, i0, k, out, n, accumulate, av);
+      i0 += 2;
+    } else {
+      k_ritz<V, 1><<<grid, 256, 0, st>>>(Vb, stride, m, Sd, Sf, ldS, i0, k, out, n, accumulate, av);
+      i0 += 1;
+    }
+  }
+  ED_LAUNCH_CHECK();
+  return ED_OK;
 }
 
 __global__ void k_step_inc(int* step) { *step += 1; }
@@ -315,9 +490,9 @@ struct Work {
 };
 
 template <class V>
-int dot_to(Work<V>& W, const V* x, const V* y, int op, int slot, double thr = 0.0) {
+int dot_to(Work<V>& W, const V* x, const V* y, int op, int slot) {
   k_dot<V><<<W.grid, kRedThreads, 0, W.st>>>(x, y, W.n, W.partial);
-  k_finish<<<1, kRedThreads, 0, W.st>>>(W.partial, (int)W.grid, op, slot, W.c, thr);
+  k_finish<<<1, kRedThreads, 0, W.st>>>(W.partial, (int)W.grid, op, slot, W.c);
   ED_LAUNCH_CHECK();
   return ED_OK;
 }
@@ -333,7 +508,7 @@ int cgs2(Work<V>& W, const V* Vb, uint64_t stride, int nvec, V* w, LzTerm<V> lz 
   const uint32_t nb = cgs_grid<V>(W.ctx, W.n);
   const LzTerm<V> none;
   auto finish = [&](int k0, int kn) {
-    k_finish<<<kn, kRedThreads, 0, W.st>>>(W.hpart, (int)nb, OP_NEGH, k0, W.c, 0.0);
+    k_finish<<<kn, kRedThreads, 0, W.st>>>(W.hpart, (int)nb, OP_NEGH, k0, W.c);
   };
   auto dots = [&](int k0, int kn, int rev, const LzTerm<V>& t) {
     k_cgs<V, false, true><<<nb, kCgsThreads, cgs_smem<V>(kn, false, true), W.st>>>(
@@ -639,7 +814,7 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
       ++restarts;
       k_random<V><<<vgrid, 256, 0, st>>>(w, n, o->seed + 7919ull * restarts);
       ED_TRY(cgs2(W, (const V*)Vbase, ld, m, w));
-      k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c, 0.0);
+      k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c);
       k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(m), n, c, 1);
       // beta[m] = 0 splits T; reset the exhaustion flag
       double zero = 0.0;
@@ -663,9 +838,7 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
     // S for the final m
     ED_TRY(tridiag(ctx, st, c, m, kc, 0.0, theta, Sd, Sf, ldS, resid, twork));
     V* out = static_cast<V*>(evecs);
-    for (int i0 = 0; i0 < kc; i0 += 8)
-      k_ritz<V, 8><<<vgrid, 256, 0, st>>>(Vbase, ld, m, Sd, Sf, ldS, i0, std::min(8, kc - i0), out, n, 0);
-    ED_LAUNCH_CHECK();
+    ED_TRY(ritz(ctx, st, (const V*)Vbase, ld, m, Sd, Sf, ldS, kc, out, n, 0));
   }
   ED_TRY_CUDA(cudaStreamSynchronize(st));
   for (int q = 0; q < n_timed; ++q) {

@@ -65,7 +65,9 @@ struct Run3 {
   Coefs c{};
   char* cbuf = nullptr;
   size_t cbytes = 0;
-  uint32_t sgrid = 0;
+  uint32_t sgrid = 0, lgrid = 0;
+  NormPart norms{{nullptr, nullptr}};
+  double thr = 0.0;
   int np_apply = 0;
   cudaGraphExec_t g[3] = {nullptr, nullptr, nullptr};
   int launched = 0;
@@ -98,7 +100,7 @@ struct Run3 {
 
   // Allocate, copy the start vector (or draw one), normalise, capture the step graphs.
   int init(Sector* sec, Ctx* cx, cudaStream_t stream, int max_steps, const V* start, uint64_t seed, int k,
-           double thr) {
+           double step_thr) {
     s = sec;
     ctx = cx;
     st = stream;
@@ -109,7 +111,11 @@ struct Run3 {
     ED_TRY(alloc(&v0, n));
     sgrid = (uint32_t)std::min<uint64_t>((n + kRedThreads - 1) / kRedThreads, (uint64_t)ctx->num_sms * 8);
     if (sgrid == 0) sgrid = 1;
-    ED_TRY(alloc(&partial, std::max<uint64_t>(sgrid, (uint64_t)ctx->num_sms * 8)));
+    const uint64_t na = std::max<uint64_t>(sgrid, (uint64_t)ctx->num_sms * 8);
+    lgrid = lz_grid(ctx, n);
+    thr = step_thr;
+    ED_TRY(alloc(&partial, na + 2 * (uint64_t)lgrid));
+    norms = NormPart{{partial + na, partial + na + lgrid}};
     cbytes = coef_bytes(mmax, std::max(k, 1)) + 8 * 1024 + (size_t)(mmax + 2) * 64 * std::max(k, 1);
     ED_TRY(alloc(&cbuf, cbytes));
     Carve cv{cbuf};
@@ -123,15 +129,14 @@ struct Run3 {
     }
     ED_TRY_CUDA(cudaMemcpyAsync(v0, Q[0], n * sizeof(V), cudaMemcpyDeviceToDevice, st));
     k_dot<V><<<sgrid, kRedThreads, 0, st>>>(Q[0], Q[0], n, partial);
-    k_finish<<<1, kRedThreads, 0, st>>>(partial, (int)sgrid, OP_SIGMA0, 0, c, 0.0);
+    k_finish<<<1, kRedThreads, 0, st>>>(partial, (int)sgrid, OP_SIGMA0, 0, c);
     ED_LAUNCH_CHECK();
     for (int ph = 0; ph < 3; ++ph) {
       cudaGraph_t graph = nullptr;
       ED_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       int r = apply_dot_launch(Q[ph], Y);
-      k_finish<<<1, kRedThreads, 0, st>>>(partial, np_apply, OP_ALPHA_Q, -1, c, 0.0);
-      k_lz_step<V><<<sgrid, kRedThreads, 0, st>>>(Y, Q[ph], Q[(ph + 2) % 3], Q[(ph + 1) % 3], n, c, -1, partial);
-      k_finish<<<1, kRedThreads, 0, st>>>(partial, (int)sgrid, OP_BETA_Q, -2, c, thr);
+      k_lz_step<V><<<lgrid, kRedThreads, 0, st>>>(Y, Q[ph], Q[(ph + 2) % 3], Q[(ph + 1) % 3], n, c, -1, partial,
+                                                 np_apply, norms, thr);
       k_step_inc<<<1, 1, 0, st>>>(c.step);
       cudaError_t ce = cudaStreamEndCapture(st, &graph);
       if (r != ED_OK) {
@@ -156,6 +161,13 @@ struct Run3 {
   int launch_step() {
     ED_TRY_CUDA(cudaGraphLaunch(g[launched % 3], st));
     ++launched;
+    return ED_OK;
+  }
+
+  // beta of the last step, ahead of reading the coefficients.
+  int close() {
+    k_lz_close<<<1, 32, 0, st>>>(norms, (int)lgrid, c, launched, thr);
+    ED_LAUNCH_CHECK();
     return ED_OK;
   }
 };
@@ -611,6 +623,7 @@ struct Server : ServerBase {
     // asynchronous convergence check: exhaustion flag, tridiagonal solve, residual
     const int m = r->launched;
     q->m_check = m;
+    ED_TRY(r->close());
     ED_TRY(tridiag(ctx, q->st, r->c, m, 1, 0.0, q->theta, q->Sd, q->Sf, r->mmax + 3, q->resid, q->twork));
     ED_TRY_CUDA(cudaMemcpyAsync(q->h_pin, q->theta, sizeof(double), cudaMemcpyDeviceToHost, q->st));
     ED_TRY_CUDA(cudaMemcpyAsync(q->h_pin + 1, q->Sd + (m - 1), sizeof(double), cudaMemcpyDeviceToHost, q->st));
@@ -673,11 +686,11 @@ struct Server : ServerBase {
     const int burst = 8;
     for (int b = 0; b < burst && q->vec_step < q->m_final; ++b) {
       const int jj = q->vec_step;
-      k_ritz<V, 8><<<vg, 256, 0, q->st>>>(r->q(jj), n, 1, q->Sq + jj, q->Sqf + jj, r->mmax + 3, 0, 1, q->psi, n, 1);
+      ED_TRY(ritz(ctx, q->st, (const V*)r->q(jj), n, 1, q->Sq + jj, q->Sqf + jj, r->mmax + 3, 1, q->psi, n, 1));
       if (jj + 1 < q->m_final) {
         ED_TRY(apply_h(q->sec.get(), r->q(jj), r->Y, q->st));
-        k_lz_step<V><<<r->sgrid, kRedThreads, 0, q->st>>>(r->Y, r->q(jj), jj > 0 ? r->q(jj - 1) : nullptr,
-                                                          r->q(jj + 1), n, r->c, jj, nullptr);
+        k_lz_regen<V><<<r->lgrid, kRedThreads, 0, q->st>>>(r->Y, r->q(jj), jj > 0 ? r->q(jj - 1) : nullptr,
+                                                           r->q(jj + 1), n, r->c, jj);
       }
       ED_LAUNCH_CHECK();
       ++q->vec_step;
@@ -686,7 +699,7 @@ struct Server : ServerBase {
     // unit norm: a ghost copy of the converged ground state (loss of
     // orthogonality, early with float vectors) leaves sum_j S_j v_j unnormalised
     k_dot<V><<<r->sgrid, kRedThreads, 0, q->st>>>(q->psi, q->psi, n, r->partial);
-    k_finish<<<1, kRedThreads, 0, q->st>>>(r->partial, (int)r->sgrid, OP_NORM_INV, 0, r->c, 0.0);
+    k_finish<<<1, kRedThreads, 0, q->st>>>(r->partial, (int)r->sgrid, OP_NORM_INV, 0, r->c);
     k_rescale<V><<<vg, 256, 0, q->st>>>(q->psi, n, r->c, 0);
     ED_LAUNCH_CHECK();
     ED_TRY_CUDA(cudaStreamSynchronize(q->st));  // r->c is freed with the ground-state run

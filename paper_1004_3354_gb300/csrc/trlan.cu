@@ -461,7 +461,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
         ++injections;
         k_random<V><<<vgrid, 256, 0, st>>>(w, n, o->seed + 7919ull * (uint64_t)injections);
         ED_TRY(cgs2(W, (const V*)Vb, ld, size, w));
-        k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c, 0.0);
+        k_finish<<<1, kRedThreads, 0, st>>>(W.partial, (int)cgs_grid<V>(ctx, n), OP_NORM_INV, 1, c);
         k_scale<V><<<vgrid, 256, 0, st>>>(w, vec(size), n, c, 1);
         ED_LAUNCH_CHECK();
         const double zero = 0.0;
@@ -487,9 +487,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
       status = ED_ERR_NOT_CONVERGED;
       break;
     }
-    for (int i0 = 0; i0 < keep; i0 += 8)
-      k_ritz<V, 8><<<vgrid, 256, 0, st>>>(Vb, ld, m, Sd, Sf, ldS, i0, std::min(8, keep - i0), T, n, 0);
-    ED_LAUNCH_CHECK();
+    ED_TRY(ritz(ctx, st, (const V*)Vb, ld, m, Sd, Sf, ldS, keep, T, n, 0));
     ED_TRY_CUDA(cudaMemcpy2DAsync(Vb, ld * eb, T, n * eb, n * eb, keep, cudaMemcpyDeviceToDevice, st));
     ED_TRY_CUDA(cudaMemcpyAsync(vec(keep), vec(m), n * eb, cudaMemcpyDeviceToDevice, st));
     k_tr_keep<<<1, 128, 0, st>>>(theta, Sd, ldS, m, keep, c, th, sv);
@@ -506,9 +504,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   if (evecs && kc > 0) {
     // Sd holds the eigenvectors of the last projected matrix (size `size`)
     V* out = static_cast<V*>(evecs);
-    for (int i0 = 0; i0 < kc; i0 += 8)
-      k_ritz<V, 8><<<vgrid, 256, 0, st>>>(Vb, ld, size, Sd, Sf, ldS, i0, std::min(8, kc - i0), out, n, 0);
-    ED_LAUNCH_CHECK();
+    ED_TRY(ritz(ctx, st, (const V*)Vb, ld, size, Sd, Sf, ldS, kc, out, n, 0));
   }
   ED_TRY_CUDA(cudaStreamSynchronize(st));
   if (info) {
