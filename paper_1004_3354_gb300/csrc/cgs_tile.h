@@ -139,18 +139,19 @@ __device__ __forceinline__ void tile_dots(const V* __restrict__ vt, uint64_t str
   }
 }
 
-// Sum of nb doubles, the same in every thread and block: the first warp sums
-// (FP64 additions of a whole block would take longer than the rest of a small
-// kernel) and the block shares the result through sh.
-__device__ __forceinline__ double block_total(const double* __restrict__ p, int nb, double* sh) {
-  if (threadIdx.x < 32) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 32) v += p[i];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) sh[0] = v;
+// Sum of nb doubles by one warp, the same in every lane.  Four sums per lane: a
+// dependent FP64 addition takes about 100 cycles, and more warps would fill the
+// FP64 pipe (20 cycles per warp instruction and SM) instead.
+__device__ __forceinline__ double warp_total(const double* __restrict__ p, int nb, int lane) {
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = lane; i < nb; i += 128) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + 32 * q < nb) v[q] += p[i + 32 * q];
   }
-  __syncthreads();
-  return sh[0];
+  double s = (v[0] + v[1]) + (v[2] + v[3]);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 
 // Three-term update w -= alpha_j v_j + beta_j v_{j-1} ahead of the first
@@ -262,12 +263,12 @@ __global__ void __launch_bounds__(kCgsThreads, 2) k_cgs(const V* __restrict__ Vb
   V* wt = reinterpret_cast<V*>(sm);                                   // two tiles of w
   A* hs = reinterpret_cast<A*>(sm + (DOT ? 2 * E * sizeof(V) : 0));   // coefficients (UPD)
   A* hsum = hs + (UPD ? nvec : 0);                                    // the block's sums (DOT)
-  __shared__ double shd[32];
   __shared__ A sha[32];
   const uint32_t t = threadIdx.x;
   if (lz.v) {
-    const double al = block_total(lz.apart, lz.na, shd);
-    if (t == 0) {   // one thread: FP64 arithmetic of a whole block takes a microsecond
+    double al = 0.0;
+    if (t < 32) al = warp_total(lz.apart, lz.na, t);
+    if (t == 0) {
       h_split(sha[0], -al);
       h_split(sha[1], lz.vp ? -*lz.beta : 0.0);
       if (blockIdx.x == 0) {

@@ -51,7 +51,7 @@ struct Rec3 {
     if (e0) ED_TRY_CUDA(cudaEventRecord(e0, W->st));
     ED_TRY(apply_dot<V>(s, *W, q(j), Y, &np));
     if (e1) ED_TRY_CUDA(cudaEventRecord(e1, W->st));
-    k_lz_step<V><<<grid(), kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,
+    k_lz_step<V><<<grid(), kLzThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j,
                                                    W->partial, np, norms(), thr);
     ED_LAUNCH_CHECK();
     return ED_OK;
@@ -65,7 +65,7 @@ struct Rec3 {
   // Regenerate q_{j+1} from q_j, q_{j-1} with the stored coefficients.
   int regen(int j) {
     ED_TRY(apply_h(s, q(j), Y, W->st));
-    k_lz_regen<V><<<grid(), kRedThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j);
+    k_lz_regen<V><<<grid(), kLzThreads, 0, W->st>>>(Y, q(j), j > 0 ? q(j - 1) : nullptr, q(j + 1), W->n, W->c, j);
     ED_LAUNCH_CHECK();
     return ED_OK;
   }

@@ -126,55 +126,63 @@ __device__ __forceinline__ A lz_combine(const V* __restrict__ y, const V* __rest
   return nacc;
 }
 
+// 1 / sqrt(v) in FP64 from a float seed and two Newton steps (8 dependent FP64
+// instructions; the library's root and division are several times that, and a
+// dependent FP64 instruction takes about 100 cycles on this chip).  v outside
+// the float range takes the library's.
+__device__ __forceinline__ double rsqrt_d(double v) {
+  const int e = __double2hiint(v);
+  if (e < (920 << 20) || e > (1140 << 20)) return 1.0 / sqrt(v);
+  double y = (double)rsqrtf((float)v);
+  const double h = -0.5 * v;
+  y = y * fma(h, y * y, 1.5);
+  return y * fma(h, y * y, 1.5);
+}
+
 // beta_j and sigma_j = 1 / beta_j from v = |q_j|^2, sc the running scale.
 __device__ __forceinline__ void lz_beta(double v, double& sc, double thr, double& beta, double& sigma, bool& dead) {
-  const double b = sqrt(fmax(v, 0.0));
+  const double y = v > 0.0 ? rsqrt_d(v) : 0.0;
+  const double b = v > 0.0 ? v * y : 0.0;
   sc = fmax(sc, b);
   dead = !(b > thr * fmax(sc, 1.0));
   beta = dead ? 0.0 : b;
-  sigma = dead ? 0.0 : 1.0 / b;
+  sigma = dead ? 0.0 : y;
 }
 
 // One three-vector step after H q_j (in y): alpha_j from the na partials of
 // <q_j, H q_j>, beta_j from the previous step's nn partials of |q_j|^2
 // (npart[(j - 1) & 1]), then q_{j+1} and the partials of its norm
-// (npart[j & 1]).  Every block forms the step's numbers itself, one warp per
-// sum and one thread for the rest, so a step is two launches (H*v and this)
+// (npart[j & 1]).  Every block forms the step's numbers itself, so a step is two launches (H*v and this)
 // where separate finishing launches made it four; block 0 keeps them.  j < 0:
 // the step index in c.step (graph replays).
+constexpr int kLzThreads = 1024;
 struct NormPart {
   double* p[2];
 };
 template <class V>
-__global__ void __launch_bounds__(kRedThreads) k_lz_step(const V* __restrict__ y, const V* __restrict__ qj,
+__global__ void __launch_bounds__(kLzThreads) k_lz_step(const V* __restrict__ y, const V* __restrict__ qj,
                                                          const V* qjm, V* qout, uint64_t n, Coefs c, int j,
                                                          const double* __restrict__ apart, int na, NormPart npart,
                                                          double thr) {
   using A = typename AccOf<V>::T;
   __shared__ A sh[32];
   __shared__ double tot[2];
+  __shared__ double ud[3];
   __shared__ A u[3];
   if (j < 0) j = *c.step;
   if (j == 0) qjm = nullptr;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (warp < 2) {
-    const double* p = warp == 0 ? apart : npart.p[(j + 1) & 1];
-    const int nb = warp == 0 ? na : (j > 0 ? (int)gridDim.x : 0);
-    double v = 0.0;
-    for (int i = lane; i < nb; i += 32) v += p[i];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) tot[warp] = v;
-  }
+  if (warp == 0) tot[0] = warp_total(apart, na, lane);
+  if (warp == 1) tot[1] = warp_total(npart.p[(j + 1) & 1], j > 0 ? (int)gridDim.x : 0, lane);
   __syncthreads();
   if (threadIdx.x == 0) {
     double sc = c.scale[j & 1], beta = 0.0, sg = c.sigma[0];
     bool dead = false;
     if (j > 0) lz_beta(tot[1], sc, thr, beta, sg, dead);
     const double a = sg * sg * tot[0];
-    const double ua = sg, ub = -a * sg, uc = j > 0 ? -beta * c.sigma[j - 1] : 0.0;
-    h_split(u[0], ua);
-    h_split(u[1], ub);
-    h_split(u[2], uc);
+    ud[0] = sg;
+    ud[1] = -a * sg;
+    ud[2] = j > 0 ? -beta * c.sigma[j - 1] : 0.0;
     if (blockIdx.x == 0) {
       if (j > 0) {
         c.beta[j] = beta;
@@ -183,12 +191,15 @@ __global__ void __launch_bounds__(kRedThreads) k_lz_step(const V* __restrict__ y
       }
       c.alpha[j] = a;
       c.scale[(j + 1) & 1] = fmax(sc, fabs(a));
-      c.ua_d[j] = ua;
-      c.ua_f[j] = df_from_double(ua);
-      c.ub_d[j] = ub;
-      c.ub_f[j] = df_from_double(ub);
-      c.uc_d[j] = uc;
-      c.uc_f[j] = df_from_double(uc);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    const int i = threadIdx.x;
+    h_split(u[i], ud[i]);
+    if (blockIdx.x == 0) {
+      (i == 0 ? c.ua_d : i == 1 ? c.ub_d : c.uc_d)[j] = ud[i];
+      (i == 0 ? c.ua_f : i == 1 ? c.ub_f : c.uc_f)[j] = df_from_double(ud[i]);
     }
   }
   __syncthreads();
@@ -216,7 +227,7 @@ __global__ void k_lz_close(NormPart npart, int nn, Coefs c, int m, double thr) {
 
 // q_{j+1} again from y = H q_j and the stored coefficients of step j.
 template <class V>
-__global__ void __launch_bounds__(kRedThreads) k_lz_regen(const V* __restrict__ y, const V* __restrict__ qj,
+__global__ void __launch_bounds__(kLzThreads) k_lz_regen(const V* __restrict__ y, const V* __restrict__ qj,
                                                           const V* qjm, V* qout, uint64_t n, Coefs c, int j) {
   using A = typename AccOf<V>::T;
   A ua, ub, uc;
@@ -226,9 +237,10 @@ __global__ void __launch_bounds__(kRedThreads) k_lz_regen(const V* __restrict__ 
   lz_combine<V, false, A>(y, qj, qjm, qout, n, ua, ub, uc);
 }
 
-// Blocks of the three-vector kernels; their norm partials take two such rows.
+// One block per SM: each sums the partials itself, and four blocks of 256
+// threads spent 2 us of FP64 pipe on that (12.6 us per step at dim 853,776).
 inline uint32_t lz_grid(const Ctx* c, uint64_t n) {
-  const uint64_t g = (n + 2 * kRedThreads - 1) / (2 * kRedThreads), most = (uint64_t)c->num_sms * 4;
+  const uint64_t g = (n + 2 * kLzThreads - 1) / (2 * kLzThreads), most = (uint64_t)c->num_sms;
   return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({g, most, 1024}));
 }
 // Norm partials in a context's reduction scratch, past the dot products' share.
@@ -268,19 +280,19 @@ __global__ void __launch_bounds__(kRedThreads) k_scale_beta(const V* __restrict_
   using A = typename AccOf<V>::T;
   using W16 = Vec16<V>;
   using VT = typename W16::T;
-  __shared__ double sh[32];
   __shared__ A inv_s;
-  const double tot = block_total(partial, nb, sh);
-  if (threadIdx.x == 0) {   // one thread: FP64 roots and divisions of a whole block would take microseconds
-    const double b = sqrt(fmax(tot, 0.0));
-    const double sc = fmax(c.scale[ph], b);
-    const bool dead = !(b > thr * fmax(sc, 1.0));
+  double tot = 0.0;
+  if (threadIdx.x < 32) tot = warp_total(partial, nb, threadIdx.x);
+  if (threadIdx.x == 0) {
+    double sc = c.scale[ph], beta, inv;
+    bool dead;
+    lz_beta(tot, sc, thr, beta, inv, dead);
+    h_split(inv_s, inv);
     if (blockIdx.x == 0) {
       c.scale[1 - ph] = sc;
       if (dead && *c.exhausted < 0) *c.exhausted = slot;
-      c.beta[slot] = dead ? 0.0 : b;
+      c.beta[slot] = beta;
     }
-    h_split(inv_s, dead ? 0.0 : 1.0 / b);
   }
   __syncthreads();
   const A inv = inv_s;

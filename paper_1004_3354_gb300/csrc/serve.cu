@@ -135,7 +135,7 @@ struct Run3 {
       cudaGraph_t graph = nullptr;
       ED_TRY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       int r = apply_dot_launch(Q[ph], Y);
-      k_lz_step<V><<<lgrid, kRedThreads, 0, st>>>(Y, Q[ph], Q[(ph + 2) % 3], Q[(ph + 1) % 3], n, c, -1, partial,
+      k_lz_step<V><<<lgrid, kLzThreads, 0, st>>>(Y, Q[ph], Q[(ph + 2) % 3], Q[(ph + 1) % 3], n, c, -1, partial,
                                                  np_apply, norms, thr);
       k_step_inc<<<1, 1, 0, st>>>(c.step);
       cudaError_t ce = cudaStreamEndCapture(st, &graph);
@@ -689,7 +689,7 @@ struct Server : ServerBase {
       ED_TRY(ritz(ctx, q->st, (const V*)r->q(jj), n, 1, q->Sq + jj, q->Sqf + jj, r->mmax + 3, 1, q->psi, n, 1));
       if (jj + 1 < q->m_final) {
         ED_TRY(apply_h(q->sec.get(), r->q(jj), r->Y, q->st));
-        k_lz_regen<V><<<r->lgrid, kRedThreads, 0, q->st>>>(r->Y, r->q(jj), jj > 0 ? r->q(jj - 1) : nullptr,
+        k_lz_regen<V><<<r->lgrid, kLzThreads, 0, q->st>>>(r->Y, r->q(jj), jj > 0 ? r->q(jj - 1) : nullptr,
                                                            r->q(jj + 1), n, r->c, jj);
       }
       ED_LAUNCH_CHECK();

@@ -123,6 +123,17 @@ __device__ inline double tri_eig_one(const double* __restrict__ a, const double*
   return 0.5 * (lo + hi) / inv;
 }
 
+// 1 / d from a float seed and two Newton steps (the library's division is a
+// chain of about twelve FP64 instructions; a dependent one takes about 100
+// cycles on this chip).  d outside the float range takes the library's.
+__device__ __forceinline__ double tri_rcp(double d) {
+  const int e = tri_exp(d);
+  if (e < (910 << 20) || e > (1130 << 20)) return 1.0 / d;
+  double y = (double)(1.0f / (float)d);
+  y = fma(y, fma(-d, y, 1.0), y);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
 // Vector of eigenvalue k = theta by inverse iteration: solve (T - theta I) x =
 // x_prev by tridiagonal Gaussian elimination with partial pivoting (row
 // interchanges as in LAPACK's gttrf/gtts2), three sweeps, one warp: lane 0 runs
@@ -153,7 +164,7 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
     for (int r = 0; r + 1 < m; ++r) {
       const double sub = dl[r], nd = x[r + 1], nu = dl[r + 1];
       if (fabs(d) >= fabs(sub)) {
-        const double f = (d != 0.0) ? sub / d : 0.0;
+        const double f = (d != 0.0) ? sub * tri_rcp(d) : 0.0;
         rd[r] = d;
         dl[r] = f;
         du[r] = u;
@@ -162,7 +173,7 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
         d = nd - f * u;
         u = nu;
       } else {
-        const double f = d / sub;
+        const double f = d * tri_rcp(sub);
         rd[r] = sub;
         dl[r] = f;
         du[r] = nd;
