@@ -89,14 +89,24 @@ constexpr int kChunkRow = 256;  // entries of one cross table row (8 sites)
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
+// Shared memory of k_apply_win: one or two row buffers (the staged row and its
+// lists), then the tables of the launch.
 template <class P>
-size_t fast_smem(uint32_t D, int n_coef, int n_lp, uint32_t lcap, int n_chunks = 0) {
+__host__ __device__ inline size_t win_tables(int n_coef) {
+  return align16(n_coef * sizeof(typename P::C)) + align16(kMaxDelta * 4);
+}
+template <class P>
+__host__ __device__ inline size_t win_row(uint32_t D, int n_lp, uint32_t lcap, int n_chunks) {
   using V = typename P::V;
   using C = typename P::C;
   const size_t nl = (size_t)n_lp * lcap;
-  return align16(D * sizeof(V)) + align16(n_coef * sizeof(C)) + align16(nl * sizeof(C)) + align16(kList * sizeof(C)) +
-         align16(nl * sizeof(int64_t)) + align16(kList * sizeof(uint64_t)) + align16(kList * 4) +
-         align16(kMaxDelta * 4) + align16((size_t)n_lp * 4) + (size_t)n_chunks * kChunkRow * sizeof(C);
+  return align16(D * sizeof(V)) + align16(nl * sizeof(C)) + align16(kList * sizeof(C)) + align16(nl * sizeof(int64_t)) +
+         align16(kList * sizeof(uint64_t)) + align16(kList * 4) + align16((size_t)n_lp * 4) +
+         align16((size_t)n_chunks * kChunkRow * sizeof(C));
+}
+template <class P>
+size_t fast_smem(uint32_t D, int n_coef, int n_lp, uint32_t lcap, int n_chunks = 0, int bufs = 1) {
+  return win_tables<P>(n_coef) + bufs * win_row<P>(D, n_lp, lcap, n_chunks);
 }
 
 // four consecutive table entries (16-byte aligned)
@@ -135,8 +145,10 @@ __device__ __forceinline__ uint32_t sel4(const uint4& v, int e) {
 }
 
 // GEN: the general diagonal (several cross-table chunks) instead of one table
-// row per up-string pattern.
-template <class P, int BS, int MINB, bool GEN = false>
+// row per up-string pattern.  DB: two row buffers; while the warps work on one
+// row the next one is copied in, and the last warp (whose windows are the
+// fewest) builds its lists before its own windows.
+template <class P, int BS, int MINB, bool GEN, bool DB>
 __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typename P::V* __restrict__ x,
                                                        typename P::V* __restrict__ y) {
   using V = typename P::V;
@@ -144,34 +156,50 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
   using C = typename P::C;
   extern __shared__ __align__(16) unsigned char sm[];
   const uint32_t D = F.D;
-  unsigned char* p = sm;
-  V* xs = reinterpret_cast<V*>(p);
-  p += align16(D * sizeof(V));
-  C* cs = reinterpret_cast<C*>(p);
-  p += align16(F.n_coef * sizeof(C));
   const uint32_t lcap = F.lcap;
   const size_t nl = (size_t)F.n_lp * lcap;
-  // term lists of the row, one per impurity pattern p (a single list without
-  // the delta layout): the up hops, then the spin-flip / pair-hop entries that
-  // apply to every down string of pattern p, with the pattern's rank shift
-  // folded into the offset and its sign into the coefficient
-  C* lc = reinterpret_cast<C*>(p);
-  p += align16(nl * sizeof(C));
-  C* mc = reinterpret_cast<C*>(p);          // mixed coefficients
-  p += align16(kList * sizeof(C));
-  int64_t* lr = reinterpret_cast<int64_t*>(p);    // element offsets of the list terms
-  p += align16(nl * sizeof(int64_t));
-  uint64_t* mr = reinterpret_cast<uint64_t*>(p);  // mixed row offsets
-  p += align16(kList * sizeof(uint64_t));
-  uint32_t* mm = reinterpret_cast<uint32_t*>(p);  // mixed move offsets
-  p += align16(kList * 4);
-  int32_t* mds = reinterpret_cast<int32_t*>(p);   // move shifts per pattern
-  p += align16(kMaxDelta * 4);
-  int* ln = reinterpret_cast<int*>(p);            // list lengths
-  p += align16((size_t)F.n_lp * 4);
-  C* ws = reinterpret_cast<C*>(p);                // the row's cross-table rows (GEN)
-  __shared__ int n_up_s, n_mx_s;
-  __shared__ uint32_t pat_s;
+  const size_t row_bytes = win_row<P>(D, F.n_lp, lcap, GEN ? F.n_chunks : 0);
+  // one row buffer: row, tables, lists; two: row, lists, row, lists, tables
+  const size_t tables = DB ? 2 * row_bytes : align16(D * sizeof(V));
+  C* cs = reinterpret_cast<C*>(sm + tables);
+  int32_t* mds = reinterpret_cast<int32_t*>(sm + tables + align16(F.n_coef * sizeof(C)));   // move shifts per pattern
+  // one row buffer: the staged row, then its term lists, one per impurity
+  // pattern p (a single list without the delta layout): the up hops, then the
+  // spin-flip / pair-hop entries that apply to every down string of pattern p,
+  // with the pattern's rank shift folded into the offset and its sign into the
+  // coefficient; the mixed entries for the windows of several patterns
+  struct Row {
+    V* xs;
+    C* lc;
+    C* mc;           // mixed coefficients
+    int64_t* lr;     // element offsets of the list terms
+    uint64_t* mr;    // mixed row offsets
+    uint32_t* mm;    // mixed move offsets
+    int* ln;         // list lengths
+    C* ws;           // the row's cross-table rows (GEN)
+  };
+  auto row_of = [&](int b) {
+    unsigned char* p = sm + (DB ? b * row_bytes : 0);
+    Row r;
+    r.xs = reinterpret_cast<V*>(p);
+    p += align16(D * sizeof(V)) + (DB ? 0 : win_tables<P>(F.n_coef));
+    r.lc = reinterpret_cast<C*>(p);
+    p += align16(nl * sizeof(C));
+    r.mc = reinterpret_cast<C*>(p);
+    p += align16(kList * sizeof(C));
+    r.lr = reinterpret_cast<int64_t*>(p);
+    p += align16(nl * sizeof(int64_t));
+    r.mr = reinterpret_cast<uint64_t*>(p);
+    p += align16(kList * sizeof(uint64_t));
+    r.mm = reinterpret_cast<uint32_t*>(p);
+    p += align16(kList * 4);
+    r.ln = reinterpret_cast<int*>(p);
+    p += align16((size_t)F.n_lp * 4);
+    r.ws = reinterpret_cast<C*>(p);
+    return r;
+  };
+  __shared__ int n_up_s[2], n_mx_s[2];
+  __shared__ uint32_t pat_s[2];
   const bool mixd = F.dpat4 != nullptr;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int NWARP = BS / 32;
@@ -181,18 +209,21 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
   for (int k = threadIdx.x; k < F.n_md; k += BS) mds[k] = F.mdelta[k];
   A dacc = P::zero();  // <x, y> over this thread's elements (only used with F.dotp)
 
-  for (uint32_t i = blockIdx.x; i < F.D_up; i += gridDim.x) {
-    const uint32_t u = F.row_order[i];
-    __syncthreads();
+  // every thread's share of the asynchronous copy of row u
+  auto stage = [&](uint32_t u, V* xs) {
     const V* xr = x + (uint64_t)u * D;
     for (uint32_t d = threadIdx.x; d < D; d += BS) cp_async_elem(xs + d, xr + d);
+  };
+  // the lists of row u, by threads t0 .. t0 + nt - 1 of which the last warp
+  // is a part (the ballots of the per-pattern lists are its own)
+  auto lists = [&](uint32_t u, int b, const Row& r, uint32_t t, uint32_t nt) {
     const uint32_t h0 = F.uh_ptr[u], nh = F.uh_ptr[u + 1] - h0;
-    for (uint32_t k = threadIdx.x; k < nh; k += BS) {
+    for (uint32_t k = t; k < nh; k += nt) {
       const int64_t off = (int64_t)F.uh_tgt[h0 + k] * D;
       const C c = P::ld(F.uh_val, F.uh_val_df, h0 + k);
       for (int q = 0; q < F.n_lp; ++q) {
-        lr[q * lcap + k] = off;
-        lc[q * lcap + k] = c;
+        r.lr[q * lcap + k] = off;
+        r.lc[q * lcap + k] = c;
       }
     }
     if (mixd && warp == NWARP - 1) {
@@ -215,25 +246,25 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
         const uint32_t base = q * lcap + nh;
         if (mda != INT_MIN) {
           const uint32_t at = base + __popc(ba & below);
-          lr[at] = ta + (mda >> 1);
-          lc[at] = (mda & 1) ? P::neg(ca) : ca;
+          r.lr[at] = ta + (mda >> 1);
+          r.lc[at] = (mda & 1) ? P::neg(ca) : ca;
         }
         if (mdb != INT_MIN) {
           const uint32_t at = base + __popc(ba) + __popc(bb & below);
-          lr[at] = tb + (mdb >> 1);
-          lc[at] = (mdb & 1) ? P::neg(cb) : cb;
+          r.lr[at] = tb + (mdb >> 1);
+          r.lc[at] = (mdb & 1) ? P::neg(cb) : cb;
         }
-        if (lane == 0) ln[q] = (int)(nh + __popc(ba) + __popc(bb));
+        if (lane == 0) r.ln[q] = (int)(nh + __popc(ba) + __popc(bb));
       }
     }
     uint32_t nm = 0;
     if (F.mx_ptr) {
       const uint32_t m0 = F.mx_ptr[u];
       nm = F.mx_ptr[u + 1] - m0;
-      for (uint32_t k = threadIdx.x; k < nm; k += BS) {
-        mr[k] = (uint64_t)F.mx_tgt[m0 + k] * D;
-        mc[k] = P::ld(F.mx_val, F.mx_val_df, m0 + k);
-        mm[k] = mixd ? (uint32_t)F.mx_mv[m0 + k] * (uint32_t)F.np : (uint32_t)F.mx_mv[m0 + k] * D;
+      for (uint32_t k = t; k < nm; k += nt) {
+        r.mr[k] = (uint64_t)F.mx_tgt[m0 + k] * D;
+        r.mc[k] = P::ld(F.mx_val, F.mx_val_df, m0 + k);
+        r.mm[k] = mixd ? (uint32_t)F.mx_mv[m0 + k] * (uint32_t)F.np : (uint32_t)F.mx_mv[m0 + k] * D;
       }
     }
     if (GEN) {
@@ -241,20 +272,56 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
       for (int c = 0; c < F.n_chunks; ++c) {
         const int nb = 1 << F.w_bits[c];
         const size_t row = F.w_off[c] + ((size_t)((su >> (8 * c)) & (nb - 1)) << F.w_bits[c]);
-        for (int k = threadIdx.x; k < nb; k += BS) ws[c * kChunkRow + k] = P::ld(F.W, F.W_df, row + k);
+        for (int k = t; k < nb; k += nt) r.ws[c * kChunkRow + k] = P::ld(F.W, F.W_df, row + k);
       }
     }
-    if (threadIdx.x == 0) {
-      n_up_s = (int)nh;
-      n_mx_s = (int)nm;
-      pat_s = GEN ? 0u : F.row_pat[u];
+    if (t == 0) {
+      n_up_s[b] = (int)nh;
+      n_mx_s[b] = (int)nm;
+      pat_s[b] = GEN ? 0u : F.row_pat[u];
     }
+  };
+
+  int buf = 0;
+  if (DB && blockIdx.x < F.D_up) {
+    __syncthreads();   // the move shifts are in place
+    const uint32_t u0 = F.row_order[blockIdx.x];
+    const Row r0 = row_of(0);
+    stage(u0, r0.xs);
+    lists(u0, 0, r0, threadIdx.x, BS);
     cp_async_wait_all();
     __syncthreads();
+  }
+  for (uint32_t i = blockIdx.x; i < F.D_up; i += gridDim.x) {
+    const uint32_t u = F.row_order[i];
+    const Row R = row_of(buf);
+    if (DB) {
+      // the other buffer's readers passed the last barrier
+      if (i + gridDim.x < F.D_up) {
+        const uint32_t un = F.row_order[i + gridDim.x];
+        const Row rn = row_of(buf ^ 1);
+        stage(un, rn.xs);
+        if (warp == NWARP - 1) lists(un, buf ^ 1, rn, lane, 32);
+      }
+    } else {
+      __syncthreads();
+      stage(u, R.xs);
+      lists(u, 0, R, threadIdx.x, BS);
+      cp_async_wait_all();
+      __syncthreads();
+    }
+    V* const xs = R.xs;
+    C* const lc = R.lc;
+    C* const mc = R.mc;
+    int64_t* const lr = R.lr;
+    uint64_t* const mr = R.mr;
+    uint32_t* const mm = R.mm;
+    int* const ln = R.ln;
+    C* const ws = R.ws;
 
     const C eu = P::ld(F.e_up, F.e_up_df, u);
-    const int nup = n_up_s, nmx = n_mx_s;
-    const C* ddr = P::ld_ptr(F.dd, F.dd_df) + (uint64_t)pat_s * NE;
+    const int nup = n_up_s[buf], nmx = n_mx_s[buf];
+    const C* ddr = P::ld_ptr(F.dd, F.dd_df) + (uint64_t)pat_s[buf] * NE;
     V* yr = y + (uint64_t)u * D;
     for (uint32_t w = warp; w < F.n_win; w += NWARP) {
       const uint32_t ent = w * 32 + lane;   // this lane's four entries
@@ -391,6 +458,11 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
           st_stream(yr + dv[e], yv);
           if (F.dotp) P::dot(dacc, xs[dv[e]], yv);
         }
+    }
+    if (DB) {
+      cp_async_wait_all();
+      __syncthreads();
+      buf ^= 1;
     }
   }
   if (F.dotp) {
@@ -875,8 +947,18 @@ template <class P, int BS, int MINB, bool GEN = false>
 int launch_fast(const Sector* s, const void* x, void* y, cudaStream_t st, double* dotp, int* nparts) {
   FastView F = make_view<P>(s);
   F.dotp = dotp;
-  size_t smem = fast_smem<P>(F.D, F.n_coef, F.n_lp, F.lcap, F.n_chunks);
-  auto kern = k_apply_win<P, BS, MINB, GEN>;
+  // Two row buffers where MINB blocks of them fit an SM (1 KB reserved per
+  // block): with few rows per block the copies' and lists' latency shows (us,
+  // one / two buffers: N_s = 12 DF64 22.2 / 20.4, N_s = 13 DF64 53.0 / 49.6,
+  // N_s = 14 DF64 176 / 171).  FP64 rows only with per-pattern lists to build:
+  // the FP64 pipe hides the rest (N_s = 12 38.2 / 36.0 with moves, 29.0 / 29.6
+  // without).
+  const size_t two = fast_smem<P>(F.D, F.n_coef, F.n_lp, F.lcap, F.n_chunks, 2);
+  const size_t per_sm_bytes = s->ctx->smem_per_sm ? s->ctx->smem_per_sm : 228 * 1024;
+  const bool db = MINB * (two + 1024) <= per_sm_bytes && two <= 220 * 1024 &&
+                  (P::prec != ED_PREC_FP64 || s->fast.mix_delta);
+  const size_t smem = db ? two : fast_smem<P>(F.D, F.n_coef, F.n_lp, F.lcap, F.n_chunks);
+  auto kern = db ? k_apply_win<P, BS, MINB, GEN, true> : k_apply_win<P, BS, MINB, GEN, false>;
   ED_TRY(smem_cap(s->ctx, kern, smem));
   int per_sm = 0;
   ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem));
@@ -982,15 +1064,38 @@ int build_fast(Sector* s) {
   const size_t smem2 = s->prec == ED_PREC_DF64 ? pair_smem<PolDF>(D, nc) : pair_smem<PolF32>(D, nc);
   const bool pair = !gen && s->prec != ED_PREC_FP64 && (uint64_t)D * 2 * vbytes < (1ull << 19) && smem2 <= 220 * 1024;
 
-  // window-local order: inside each window of 128 ranks, longest hop list first
-  const uint32_t n_win = (D + kWin - 1) / kWin;
+  // Windows: runs of at most 128 consecutive ranks.  With the delta layout the
+  // down strings come in blocks of equal impurity pattern, and a window inside
+  // one block gathers its spin-flip / pair-hop terms with the up hops, while one
+  // that spans blocks walks the row's entries one round trip at a time, which
+  // costs about 0.4 of a window more (N_s = 15: 33 us of 600 for 7 of 51
+  // windows).  So the windows start anew at each block where that pays for the
+  // extra windows: N_s = 12 (8 windows either way, seven of them across blocks)
+  // and 13 (15 against 14, seven across), not N_s = 15 (56 against 51).
+  std::vector<uint32_t> dbas(D), wstart;
+  ED_TRY_CUDA(cudaMemcpy(dbas.data(), s->dn.basis, sizeof(uint32_t) * D, cudaMemcpyDeviceToHost));
+  auto pat_of = [&](uint32_t d) { return mix_delta ? dbas[d] >> s->orb0 : 0u; };
+  {
+    std::vector<uint32_t> fixed, cut;
+    uint32_t across = 0;
+    for (uint32_t d = 0; d < D; ++d) {
+      if (d % kWin == 0) fixed.push_back(d);
+      if (cut.empty() || d - cut.back() == kWin || pat_of(d) != pat_of(d - 1)) cut.push_back(d);
+    }
+    for (uint32_t w : fixed) across += pat_of(w) != pat_of(std::min(D, w + kWin) - 1) ? 1u : 0u;
+    wstart = 10 * cut.size() < 10 * fixed.size() + 4 * across ? cut : fixed;
+  }
+  const uint32_t n_win = (uint32_t)wstart.size();
+  wstart.push_back(D);
+
+  // window-local order: inside each window, longest hop list first
   std::vector<uint32_t> dptr(D + 1);
   ED_TRY_CUDA(cudaMemcpy(dptr.data(), s->dn.hop_ptr, sizeof(uint32_t) * (D + 1), cudaMemcpyDeviceToHost));
   std::vector<uint32_t> perm((size_t)n_win * kWin, D);
   std::vector<uint8_t> cnt((size_t)n_win * 4, 0);
   for (uint32_t w = 0; w < n_win; ++w) {
     std::vector<uint32_t> ds;
-    for (uint32_t d = w * kWin; d < std::min(D, (w + 1) * kWin); ++d) ds.push_back(d);
+    for (uint32_t d = wstart[w]; d < wstart[w + 1]; ++d) ds.push_back(d);
     std::stable_sort(ds.begin(), ds.end(), [&](uint32_t a, uint32_t b) {
       return (dptr[a + 1] - dptr[a]) > (dptr[b + 1] - dptr[b]);
     });
@@ -1069,14 +1174,9 @@ int build_fast(Sector* s) {
   if (gen) ED_TRY(sector_alloc(s, &f.gpat, NE));
   if (mix_delta) {
     const int M = s->M, NP = 1 << M;
-    std::vector<uint32_t> dbas(D), wpat(n_win, 0xffffffffu);
-    ED_TRY_CUDA(cudaMemcpy(dbas.data(), s->dn.basis, sizeof(uint32_t) * D, cudaMemcpyDeviceToHost));
-    for (uint32_t w = 0; w < n_win; ++w) {
-      uint32_t p0 = dbas[w * kWin] >> s->orb0;
-      bool same = true;
-      for (uint32_t d = w * kWin; d < std::min(D, (w + 1) * kWin); ++d) same = same && ((dbas[d] >> s->orb0) == p0);
-      if (same) wpat[w] = p0;
-    }
+    std::vector<uint32_t> wpat(n_win, 0xffffffffu);
+    for (uint32_t w = 0; w < n_win; ++w)   // patterns ascend with the rank
+      if (pat_of(wstart[w]) == pat_of(wstart[w + 1] - 1)) wpat[w] = pat_of(wstart[w]);
     ED_TRY(sector_alloc(s, &f.wpat, n_win));
     ED_TRY_CUDA(cudaMemcpy(f.wpat, wpat.data(), sizeof(uint32_t) * n_win, cudaMemcpyHostToDevice));
     ED_TRY(sector_alloc(s, &f.dpat, NE));

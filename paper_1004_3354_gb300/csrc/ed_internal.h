@@ -180,16 +180,17 @@ struct Sector {
   int32_t* dn_move = nullptr;
   // tables of the fast row kernel (apply_fast.cu); fast.ok = false -> generic kernels
   struct Fast {
-    // Window layout: the down strings are cut into windows of 128 consecutive
-    // ranks; inside a window they are sorted by hop count (longest first) and
-    // dealt to 32 lanes x 4 slots, entry index w*128 + lane*4 + slot.
+    // Window layout: the down strings are cut into windows of at most 128
+    // consecutive ranks (build_fast says where); inside a window they are sorted
+    // by hop count (longest first) and dealt to 32 lanes x 4 slots, entry index
+    // w*128 + lane*4 + slot.
     bool ok = false;
     // models whose interaction window spans several 8-site chunks (a Hubbard
     // cluster of more than eight sites): the one-row kernel with the general
     // diagonal; such a sector has nothing to tune
     bool gen_ok = false;
     uint32_t* gpat = nullptr;   // [n_win*128] window bits of each entry (gen_ok)
-    uint32_t n_win = 0;         // ceil(D_dn / 128)
+    uint32_t n_win = 0;
     uint32_t max_cnt = 0;       // widest down-hop list
     int n_coef = 0;             // distinct down-hop matrix elements (<= 256), one of them 0.0
     int n_pat = 1;              // 2^K diagonal patterns of the up string
