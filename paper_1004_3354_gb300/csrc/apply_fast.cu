@@ -863,20 +863,26 @@ __global__ void k_win_tables(uint32_t D, uint32_t n_win, uint32_t max_cnt, const
 }
 
 // Rank shift of each impurity move (x -> y) for each pattern p, read off the
-// move table at one string of pattern p (the shift is the same for every
-// string of the pattern when the orbitals are the top sites); INT_MIN where
-// the move does not apply.
+// move table at the first string of pattern p (the shift is the same for every
+// string of the pattern when the orbitals are the top sites: their bits lead the
+// ascending order, so a binary search finds it); INT_MIN where the move does
+// not apply.
 __global__ void k_mix_delta(uint32_t D, const uint32_t* __restrict__ dbasis, const int32_t* __restrict__ mv,
                             int orb0, int M, int32_t* __restrict__ mdelta) {
   const int NP = 1 << M;
   for (int idx = threadIdx.x; idx < M * M * NP; idx += blockDim.x) {
-    const int move = idx / NP, p = idx % NP;
+    const int move = idx / NP;
+    const uint32_t p = (uint32_t)(idx % NP);
+    uint32_t lo = 0, hi = D;   // first string whose impurity bits are at least p
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) / 2;
+      if ((dbasis[mid] >> orb0) < p) lo = mid + 1;
+      else hi = mid;
+    }
     int32_t out = INT_MIN;
-    for (uint32_t d = 0; d < D; ++d) {
-      if ((int)(dbasis[d] >> orb0) != p) continue;
-      const int32_t v = mv[(uint64_t)move * D + d];
-      if (v >= 0) out = (int32_t)(((int64_t)(v >> 1) - (int64_t)d) * 2 + (v & 1));
-      break;
+    if (lo < D && (dbasis[lo] >> orb0) == p) {
+      const int32_t v = mv[(uint64_t)move * D + lo];
+      if (v >= 0) out = (int32_t)(((int64_t)(v >> 1) - (int64_t)lo) * 2 + (v & 1));
     }
     mdelta[idx] = out;
   }

@@ -23,8 +23,19 @@ namespace ed {
 
 namespace {
 
-// 1 / (c + i d) by Smith's (1962) scaled division.
+// 1 / (c + i d).  Where the squares stay well inside a double's (and a float's)
+// range, conj / |.|^2 with a reciprocal from a float seed and two Newton steps
+// (a chain of 9 dependent FP64 instructions, which take about 100 cycles each on
+// this chip); otherwise Smith's (1962) scaled division, a chain of about 27.
 __device__ __forceinline__ double2 crecip(double c, double d) {
+  const double q = fma(c, c, d * d);
+  const int e = __double2hiint(q) & 0x7ff00000;
+  if (e > (920 << 20) && e < (1120 << 20)) {
+    double y = (double)(1.0f / (float)q);
+    y = fma(y, fma(-q, y, 1.0), y);
+    y = fma(y, fma(-q, y, 1.0), y);
+    return make_double2(c * y, -d * y);
+  }
   if (fabs(c) >= fabs(d)) {
     double r = d / c, den = c + d * r;
     return make_double2(1.0 / den, -r / den);
@@ -60,6 +71,10 @@ __global__ void k_cf_accum(double2* __restrict__ G, int n_w, double beta, const 
   G[n].y += w * n2 * g.y;
 }
 
+// One warp per block: a frequency is one chain of FP64 instructions, and two
+// warps on an SM already share its FP64 pipe.
+constexpr int kCfThreads = 32;
+
 struct SectorCache {
   Ctx* ctx;
   const ed_model* m;
@@ -93,7 +108,7 @@ struct SectorCache {
 // Add one (state, part) continued fraction to G on `st` (used by the server).
 int greens_accumulate(double2* dG, int n_w, double beta, const double* da, const double* db, int L, double n2,
                       const double* dE, int n_states, int nu, int sgn, cudaStream_t st) {
-  k_cf_accum<<<(n_w + 127) / 128, 128, 0, st>>>(dG, n_w, beta, da, db, L, n2, dE, n_states, nu, sgn, nullptr);
+  k_cf_accum<<<(n_w + kCfThreads - 1) / kCfThreads, kCfThreads, 0, st>>>(dG, n_w, beta, da, db, L, n2, dE, n_states, nu, sgn, nullptr);
   ED_LAUNCH_CHECK();
   return ED_OK;
 }
@@ -172,7 +187,7 @@ int greens_cf_run(Ctx* ctx, const ed_model* m, int prec, int n_states, const ed_
         if (L > 0 && n2 > 0.0) {
           ED_TRY_CUDA(cudaMemcpyAsync(dab, ha.data(), sizeof(double) * depth, cudaMemcpyHostToDevice, st));
           ED_TRY_CUDA(cudaMemcpyAsync(dab + depth, hb.data(), sizeof(double) * depth, cudaMemcpyHostToDevice, st));
-          k_cf_accum<<<(n_w + 127) / 128, 128, 0, st>>>(dG, n_w, beta, dab, dab + depth, L, n2, dE, n_states, nu,
+          k_cf_accum<<<(n_w + kCfThreads - 1) / kCfThreads, kCfThreads, 0, st>>>(dG, n_w, beta, dab, dab + depth, L, n2, dE, n_states, nu,
                                                        dag ? 1 : -1, dz);
           ED_LAUNCH_CHECK();
           ED_TRY_CUDA(cudaStreamSynchronize(st));  // ha/hb are reused
