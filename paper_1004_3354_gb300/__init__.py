@@ -213,14 +213,24 @@ def _ptr(t):
     """Address of a torch tensor's or numpy array's data (None stays NULL)."""
     if t is None:
         return None
-    return C.c_void_p(t.data_ptr() if hasattr(t, "data_ptr") else t.ctypes.data)
+    return t.data_ptr() if hasattr(t, "data_ptr") else t.ctypes.data   # c_void_p arguments take integers
+
+
+_raw_stream = None
 
 
 def _stream(stream):
-    if stream is None:
+    """cudaStream_t of a torch stream, or of the current device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
+    global _raw_stream
+    if _raw_stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        torch.cuda.init()
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # no Stream object: 0.3 us against 2.8 us
+        dev = torch.cuda.current_device
+        _raw_stream = (lambda: raw(dev())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
 
 
 # ------------------------------------------------------------------ model
