@@ -127,7 +127,7 @@ typedef struct ed_sector_info {
   uint64_t csr_nnz;             /* stored CSR entries (0 without ED_SECTOR_CSR) */
   uint64_t table_bytes;         /* device bytes held by the sector */
   double   nnz_per_row;         /* mean stored entries per row of H (diagonal included) */
-  int      kernel;              /* H*v kernel in use: 0 flat, 1 row-staged generic, 2 fast row
+  int      kernel;              /* H*v kernel in use: 0 flat, 1 row-staged (general models), 2 fast row
                                    kernel, 3 fast two-row kernel (DF64 when the autotuner picks
                                    it; FP32 where 4 does not apply), 4 natural-order float kernel
                                    (the FP32 default) */

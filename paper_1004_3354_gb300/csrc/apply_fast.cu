@@ -9,7 +9,7 @@
 //    counts on each bond-connected cluster of sites), so the x rows that the
 //    up hops of concurrently processed rows read stay resident in L2.
 //  * A block stages one x row in shared memory (cp.async) and its warps sweep
-//    the row in windows of 128 consecutive down strings.  Inside a window the
+//    the row in windows of at most 128 consecutive down strings.  Inside a window the
 //    strings are sorted by hop count and dealt to 32 lanes x 4 slots, so the
 //    lanes of a warp run the same number of down hops per slot, every global
 //    access of the warp stays inside the window's 128 elements, and each thread
@@ -26,6 +26,10 @@
 //    pattern, with the shift folded into the offset and the sign into the
 //    coefficient.  A window whose strings share one pattern (most of them)
 //    then gathers all its global terms in one loop, two at a time.
+//  * Rows short enough for two buffers are copied in and listed while the warps
+//    work on the row before.
+//  * Models with more than eight interacting sites use the same kernel with the
+//    general diagonal (GEN): the up string's cross-table rows, staged per row.
 #include <algorithm>
 #include <climits>
 #include <functional>
