@@ -12,6 +12,7 @@
 
 #include "cgs_tile.h"
 #include "ed_internal.h"
+#include "fp64_short.h"
 #include "tri_common.h"
 #include "vec_ops.h"
 
@@ -126,23 +127,10 @@ __device__ __forceinline__ A lz_combine(const V* __restrict__ y, const V* __rest
   return nacc;
 }
 
-// 1 / sqrt(v) in FP64 from a float seed and two Newton steps (8 dependent FP64
-// instructions; the library's root and division are several times that, and a
-// dependent FP64 instruction takes about 100 cycles on this chip).  v outside
-// the float range takes the library's.
-__device__ __forceinline__ double rsqrt_d(double v) {
-  const int e = __double2hiint(v);
-  if (e < (920 << 20) || e > (1140 << 20)) return 1.0 / sqrt(v);
-  double y = (double)rsqrtf((float)v);
-  const double h = -0.5 * v;
-  y = y * fma(h, y * y, 1.5);
-  return y * fma(h, y * y, 1.5);
-}
-
 // beta_j and sigma_j = 1 / beta_j from v = |q_j|^2, sc the running scale.
 __device__ __forceinline__ void lz_beta(double v, double& sc, double thr, double& beta, double& sigma, bool& dead) {
-  const double y = v > 0.0 ? rsqrt_d(v) : 0.0;
-  const double b = v > 0.0 ? v * y : 0.0;
+  double b = 0.0, y = 0.0;
+  if (v > 0.0) root_inverse(v, b, y);
   sc = fmax(sc, b);
   dead = !(b > thr * fmax(sc, 1.0));
   beta = dead ? 0.0 : b;

@@ -54,15 +54,12 @@ __device__ __forceinline__ void jac_cs(float t, float& c, float& s) {
   c = rsqrtf(1.f + t * t);
   s = t * c;
 }
-// cosine and sine of a given tangent to FP64 accuracy: two Newton steps from a
-// float reciprocal root (c^2 + s^2 = 1 is what keeps the vectors orthogonal)
+// cosine and sine of a given tangent to FP64 accuracy (c^2 + s^2 = 1 is what
+// keeps the vectors orthogonal)
 __device__ __forceinline__ void jac_cs(double t, double& c, double& s) {
-  const double d = fma(t, t, 1.0);
-  double y = (double)rsqrtf((float)d);
-  y = y * fma(-0.5 * d, y * y, 1.5);
-  y = y * fma(-0.5 * d, y * y, 1.5);
-  c = y;
-  s = t * y;
+  double root;
+  root_inverse(fma(t, t, 1.0), root, c);
+  s = t * c;
 }
 
 // Rotations of one round, by the first np threads: pair i of round r in the
