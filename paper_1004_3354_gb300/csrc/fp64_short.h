@@ -35,4 +35,15 @@ __device__ __forceinline__ void root_inverse(double v, double& root, double& inv
   inv = fma(fma(-root, y, 1.0), y, y);
 }
 
+// a / d from y, the reciprocal of d to 2^-46.
+__device__ __forceinline__ double quot_step(double a, double d, double y) {
+  const double g = a * y;
+  return fma(fma(-d, g, a), y, g);
+}
+// Reciprocal of d to 2^-46, d in float_range.
+__device__ __forceinline__ double rcp_seed(double d) {
+  const double y = (double)(1.0f / (float)d);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
 }  // namespace ed
