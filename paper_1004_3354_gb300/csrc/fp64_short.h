@@ -46,4 +46,9 @@ __device__ __forceinline__ double rcp_seed(double d) {
   return fma(y, fma(-d, y, 1.0), y);
 }
 
+// a / d for |a| <= |d|.
+__device__ __forceinline__ double quotient(double a, double d) {
+  return float_range(d) ? quot_step(a, d, rcp_seed(d)) : a / d;
+}
+
 }  // namespace ed

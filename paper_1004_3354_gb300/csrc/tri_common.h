@@ -13,6 +13,7 @@
 #pragma once
 
 #include "ed_internal.h"
+#include "fp64_short.h"
 
 namespace ed {
 
@@ -123,31 +124,24 @@ __device__ inline double tri_eig_one(const double* __restrict__ a, const double*
   return 0.5 * (lo + hi) / inv;
 }
 
-// 1 / d from a float seed and two Newton steps (the library's division is a
-// chain of about twelve FP64 instructions; a dependent one takes about 100
-// cycles on this chip).  d outside the float range takes the library's.
-__device__ __forceinline__ double tri_rcp(double d) {
-  const int e = tri_exp(d);
-  if (e < (910 << 20) || e > (1130 << 20)) return 1.0 / d;
-  double y = (double)(1.0f / (float)d);
-  y = fma(y, fma(-d, y, 1.0), y);
-  return fma(y, fma(-d, y, 1.0), y);
-}
-
 // Vector of eigenvalue k = theta by inverse iteration: solve (T - theta I) x =
 // x_prev by tridiagonal Gaussian elimination with partial pivoting (row
 // interchanges as in LAPACK's gttrf/gtts2), three sweeps, one warp: lane 0 runs
 // the recurrences, all lanes the rest.  wk holds 6 * m doubles of scratch.
-// Output s[j], j < m, normalised, largest entry positive.
+// Output s[j], j < m, normalised, largest entry positive.  Quotients are rounded
+// once: the factor's by a residual step; the back substitution's, by a pivot known
+// ahead, as a product with the pivot's reciprocal in two parts (one dependent
+// instruction more than with the rounded reciprocal, whose vectors have residuals
+// 6% larger).  The low part's last bit holds the row's interchange.
 __device__ inline void tri_vec_one(const double* __restrict__ a, const double* __restrict__ b, int m, double th, int k,
                                    double* wk, double* __restrict__ s) {
   const int lane = threadIdx.x;
   double* x = wk;
   double* dl = x + m;
-  double* rd = dl + m;     // pivots, then their reciprocals
+  double* rd = dl + m;     // pivots, then the high parts of their reciprocals
   double* du = rd + m;
   double* du2 = du + m;
-  double* piv = du2 + m;
+  double* rl = du2 + m;    // interchanges, then with them the low parts
   double anorm = 0.0;
   for (int r = lane; r < m; r += 32) {
     const double off = (r > 0 ? fabs(b[r]) : 0.0) + (r + 1 < m ? fabs(b[r + 1]) : 0.0);
@@ -164,33 +158,36 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
     for (int r = 0; r + 1 < m; ++r) {
       const double sub = dl[r], nd = x[r + 1], nu = dl[r + 1];
       if (fabs(d) >= fabs(sub)) {
-        const double f = (d != 0.0) ? sub * tri_rcp(d) : 0.0;
+        const double f = (d != 0.0) ? quotient(sub, d) : 0.0;
         rd[r] = d;
         dl[r] = f;
         du[r] = u;
         du2[r] = 0.0;
-        piv[r] = 0.0;
+        rl[r] = __longlong_as_double(0ll);
         d = nd - f * u;
         u = nu;
       } else {
-        const double f = d * tri_rcp(sub);
+        const double f = quotient(d, sub);
         rd[r] = sub;
         dl[r] = f;
         du[r] = nd;
         du2[r] = nu;
-        piv[r] = 1.0;
+        rl[r] = __longlong_as_double(1ll);
         d = u - f * nd;
         u = -f * nu;
       }
     }
     rd[m - 1] = d;
-    du[m - 1] = du2[m - 1] = piv[m - 1] = 0.0;
+    du[m - 1] = du2[m - 1] = rl[m - 1] = 0.0;
   }
   __syncwarp();
   for (int r = lane; r < m; r += 32) {
     double d = rd[r];
     if (fabs(d) < tiny) d = (d < 0 ? -tiny : tiny);
-    rd[r] = 1.0 / d;
+    const double y = 1.0 / d;
+    rd[r] = y;
+    rl[r] = __longlong_as_double((__double_as_longlong(fma(-d, y, 1.0) * y) & ~1ll) |
+                                 (__double_as_longlong(rl[r]) & 1ll));
     x[r] = 1.0 + 0.01 * (double)((r * 7919 + k * 104729) % 97) / 97.0;
   }
   __syncwarp();
@@ -200,16 +197,17 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
 #pragma unroll 4
       for (int r = 0; r + 1 < m; ++r) {
         const double xn = x[r + 1], f = dl[r];
-        const bool pv = piv[r] != 0.0;
+        const bool pv = __double2loint(rl[r]) & 1;
         const double keep = pv ? xn : t, go = pv ? t : xn;
         x[r] = keep;
         t = go - f * keep;
       }
-      double x1 = t * rd[m - 1], x2 = 0.0;
+      double x1 = fma(t, rd[m - 1], t * rl[m - 1]), x2 = 0.0;
       x[m - 1] = x1;
 #pragma unroll 4
       for (int r = m - 2; r >= 0; --r) {
-        const double v = (x[r] - du2[r] * x2 - du[r] * x1) * rd[r];
+        const double num = x[r] - du2[r] * x2 - du[r] * x1;
+        const double v = fma(num, rd[r], num * rl[r]);
         x[r] = v;
         x2 = x1;
         x1 = v;
@@ -219,7 +217,7 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
     double mx = 0.0;
     for (int r = lane; r < m; r += 32) mx = fmax(mx, fabs(x[r]));
     mx = tri_warp_max(mx);
-    double inv = mx > 0 ? 1.0 / mx : 0.0;
+    double inv = tri_pow2_inv(tri_exp(mx));   // to about 1, exactly
     double nrm = 0.0;
     for (int r = lane; r < m; r += 32) {
       const double v = x[r] * inv;
