@@ -71,7 +71,7 @@ struct NatDF {
   using A = float2;
   __device__ static __forceinline__ A zero() { return make_float2(0.f, 0.f); }
   __device__ static __forceinline__ C czero() { return make_float2(0.f, 0.f); }
-  __device__ static __forceinline__ void mac(A& a, C c, V x) { df_mac(a, c, x); }
+  __device__ static __forceinline__ void mac(A& a, C c, V x) { df_mac_row(a, c, x); }
   __device__ static __forceinline__ V fin(A a, A b) { return df_add(a, b); }
   __device__ static __forceinline__ void dot(float2& d, V x, V y) { df_mac(d, x, y); }
 };
