@@ -225,8 +225,9 @@ __device__ inline void tri_vec_one(const double* __restrict__ a, const double* _
       nrm += v * v;
     }
     for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
-    inv = nrm > 0 ? 1.0 / sqrt(nrm) : 0.0;
-    for (int r = lane; r < m; r += 32) x[r] *= inv;
+    const double root = sqrt(nrm);
+    inv = nrm > 0 ? 1.0 / root : 0.0;
+    for (int r = lane; r < m; r += 32) x[r] = quot_step(x[r], root, inv);   // rounded once: a single entry is 1
     __syncwarp();
   }
   // first entry of the largest magnitude positive
