@@ -197,13 +197,12 @@ __global__ void __launch_bounds__(kLzThreads) k_lz_step(const V* __restrict__ y,
 }
 
 // beta_m, sigma_m and the exhaustion flag after m steps (m < 0: c.step), ahead of
-// a convergence check; the next step forms the same numbers again.  One warp.
+// a convergence check; the next step forms the same numbers again, from the same
+// sums in the same order.  One warp.
 __global__ void k_lz_close(NormPart npart, int nn, Coefs c, int m, double thr) {
   if (m < 0) m = *c.step;
   if (m < 1) return;
-  double v = 0.0;
-  for (int i = threadIdx.x; i < nn; i += 32) v += npart.p[(m + 1) & 1][i];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const double v = warp_total(npart.p[(m + 1) & 1], nn, threadIdx.x);
   if (threadIdx.x != 0) return;
   double sc = c.scale[m & 1], beta, sg;
   bool dead;

@@ -4,6 +4,7 @@ import pytest
 import scipy.sparse.linalg as sla
 
 import workloads as W
+from oracle import greens as og
 from oracle import sector as osec
 from tests._gpu import ensure_built, torch_cuda
 
@@ -17,6 +18,28 @@ def env():
     ctx = ed.ed_ctx_create(0)
     yield ed, ctx, torch
     ed.ed_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_s", [9, 10, 11, 12, 13])   # norm partials of 7 to 152 blocks
+def test_check_and_next_step_form_the_same_beta(env, n_s):
+    """beta_1 of the three-vector recurrence as a check after one step reads it (the
+    residual of a 1 x 1 problem) and as the second step forms it (the continued
+    fraction's coefficients, the same start vector): the same bits."""
+    ed, ctx, torch = env
+    m = W.aim(n_s, seed=2)
+    nu, nd, depth = n_s // 2 - 1, n_s // 2, 3
+    C, (tu, td) = og.op_matrix(n_s, nu, nd, m.orb0, 0, True)
+    sec = ed.ed_sector_create(ctx, m, tu, td, "fp64")
+    try:
+        for seed in range(4):
+            x = W.random_vector(C.shape[1], seed=seed)
+            _, co = ed.ed_greens_cf(ctx, m, "fp64", [(nu, nd, -1.0, torch.from_numpy(x).cuda())], 40.0, 1,
+                                    orbital=m.orb0, depth=depth, want_coeffs=True)
+            _, info, _ = ed.ed_lanczos(sec, k=1, tol=1e-300, max_iter=1, check_every=1, reorth=False,
+                                       v0=torch.from_numpy(C @ x).cuda(), allow_not_converged=True)
+            assert info.residual[0] == co[0][2 + depth + 1], (seed, info.residual[0], co[0][2 + depth + 1])
+    finally:
+        ed.ed_sector_destroy(sec)
 
 
 def test_rotations_of_the_projected_matrix_have_no_bias(env):
