@@ -150,11 +150,22 @@ __device__ __forceinline__ void jac_rotate(T* A, T* Y, int ld, int mp, const uin
 // off-diagonals of about 1e-6 (two sweeps) to the same criterion as sweeps in
 // FP64 throughout.
 //
+// The float sweeps work on the matrix less its mean diagonal, scaled to entries of
+// at most 1: what float resolves follows the spread of the values, not how far
+// from zero they lie.
+//
 // k > 0: a convergence check whose decomposition is not used further.  It ends
 // after the float sweeps (110 us instead of 490 us) if one of the k lowest pairs
-// is clearly not converged, beta |s_last| above twice tol max(1, |theta|) by
-// more than 1e-3 beta (the float vectors' error; some 5e-4 at gaps of 0.05),
-// with the k lowest float values and last components as the estimates.
+// is clearly not converged: beta |s_last| above twice tol max(1, |theta|) by more
+// than beta times an estimate of the float component's error, with the k lowest
+// float values and last components as the estimates.  To first order vector i
+// takes up vector j by (what the sweeps leave at (i, j) + their rounding) / (their
+// values' distance), so the estimate is the sum of that times |s_last| of j, and at
+// least 1e-3; the rounding of some 10 m rotations of a row, 2^-24 each, is spread
+// over the matrix (three times its mean square is taken).  A pair whose neighbour
+// float cannot tell apart is not called open here, so that a check costs products
+// only where it is open (values 2^14 from zero took 88 products instead of 44 with
+// the 1e-3 alone).
 __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __restrict__ Ain, int m, int lda,
                                                             double* __restrict__ theta, double* S,
                                                             float2* __restrict__ Sf, int ldS, double* Yg,
@@ -191,28 +202,33 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
   for (int i = warp; i < np; i += nw)
     for (int j = lane; j < np; j += 32)
       if (j >= i) tab[i * np - i * (i - 1) / 2 + (j - i)] = (uint16_t)(i << 8 | j);
-  double fro = 0.0, amax = 0.0;
+  double mid = 0.0;
+  for (int i = tid; i < m; i += nt) mid += Ain[(size_t)i * lda + i];
+  mid = block_sum(mid) / (double)m;
+  double fro = 0.0, frof = 0.0, amax = 0.0;   // Frobenius norm, and that of the shifted matrix
   for (int i = warp; i < m; i += nw)
     for (int j = lane; j < m; j += 32) {
-      const double v = Ain[(size_t)i * lda + j];
+      const double v = Ain[(size_t)i * lda + j], u = i == j ? v - mid : v;
       fro += v * v;
-      amax = fmax(amax, fabs(v));
+      frof += u * u;
+      amax = fmax(amax, fabs(u));
     }
   fro = block_sum(fro);
+  frof = block_sum(frof);
   for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   if (lane == 0) red[warp] = amax;
   __syncthreads();
   for (int w = 0; w < nw; ++w) amax = fmax(amax, red[w]);
   __syncthreads();
-  // ---- float sweeps on the matrix scaled to entries of at most 1
+  // ---- float sweeps on the shifted matrix scaled to entries of at most 1
   const double inv = amax > 0.0 ? 1.0 / amax : 0.0;
   for (int i = warp; i < mp; i += nw)
     for (int j = lane; j < mp; j += 32) {
-      Af[i * ld + j] = (i < m && j < m) ? (float)(Ain[(size_t)i * lda + j] * inv) : 0.f;
+      Af[i * ld + j] = (i < m && j < m) ? (float)((Ain[(size_t)i * lda + j] - (i == j ? mid : 0.0)) * inv) : 0.f;
       Yf[i * ld + j] = i == j ? 1.f : 0.f;
     }
   __syncthreads();
-  const double frof = fro * inv * inv;
+  frof *= inv * inv;
   for (int sweep = 0; sweep < 12 && m > 1; ++sweep) {
     float off = 0.f;
     for (int i = warp; i < m; i += nw)
@@ -231,18 +247,24 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
     if (tid == 0) open = 0;
     __syncthreads();
     const double b = *beta;
+    const float E = (float)(3.0 * sqrt(10.0 / m) * 0x1p-24 * sqrt(frof));
     for (int i = tid; i < m; i += nt) {
       const float key = Af[i * ld + i];
       int at = 0;
+      float err = 0.f;
       for (int j = 0; j < m; ++j) {
         const float o = Af[j * ld + j];
         at += (o < key || (o == key && j < i)) ? 1 : 0;
+        if (j != i) {
+          const float e = fabsf(Af[i * ld + j]) + E, gap = fabsf(o - key);
+          err += e < 0.5f * gap ? e / gap * fabsf(Yf[j * ld + m - 1]) : 1.f;
+        }
       }
       if (at < k) {
-        const double th = (double)key * amax, last = fabs((double)Yf[i * ld + m - 1]);
+        const double th = fma((double)key, amax, mid), last = fabs((double)Yf[i * ld + m - 1]);
         theta[at] = th;
         S[(size_t)at * ldS + m - 1] = last;
-        if (b * (last - 1e-3) > 2.0 * tol * fmax(1.0, fabs(th))) open = 1;
+        if (b * (last - fmax(1e-3, (double)err)) > 2.0 * tol * fmax(1.0, fabs(th))) open = 1;
       }
     }
     __syncthreads();

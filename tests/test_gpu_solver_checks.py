@@ -42,6 +42,35 @@ def test_check_and_next_step_form_the_same_beta(env, n_s):
         ed.ed_sector_destroy(sec)
 
 
+@pytest.mark.parametrize("name,mk,nu,nd", [("impurity", lambda: W.aim(8, seed=4), 4, 3),
+                                           ("kanamori", lambda: W.kanamori(8, seed=4), 4, 3),
+                                           ("ring", lambda: W.hubbard_cluster(8, U=4.0, tp=0.1), 4, 4)])
+@pytest.mark.parametrize("offset", ["none", "shift", "strong U"])
+def test_restarted_checks_see_convergence_in_time(env, name, mk, nu, nd, offset):
+    """A thick restart whose basis never fills builds the Krylov space of the plain
+    solver, so its checks find the k lowest pairs converged after the same number
+    of products, rounded up to the check interval: also where the eigenvalues lie
+    far from zero or far apart beside the gaps of the wanted ones."""
+    ed, ctx, torch = env
+    m = mk()
+    if offset == "shift":       # 2^14 per electron
+        m.T = m.T + 2.0 ** 14 * np.eye(m.n_s)
+    elif offset == "strong U":
+        m.U_site = m.U_site + 2.0 ** 12 * (m.U_site != 0)
+    every = 4
+    sec = ed.ed_sector_create(ctx, m, nu, nd, "fp64")
+    try:
+        for k in (1, 2, 4):
+            for tol in (1e-10, 1e-13):
+                _, full, _ = ed.ed_lanczos(sec, k=k, tol=tol, max_iter=124, check_every=every, seed=3,
+                                           allow_not_converged=True)
+                _, tr, _ = ed.ed_lanczos_tr(sec, k=k, tol=tol, max_basis=128, max_iter=124, check_every=every, seed=3,
+                                            allow_not_converged=True)
+                assert tr.restarts == 0 and tr.iters <= -(-full.iters // every) * every, (k, tol, full.iters, tr.iters)
+    finally:
+        ed.ed_sector_destroy(sec)
+
+
 def test_rotations_of_the_projected_matrix_have_no_bias(env):
     """Values after some 200 rotations of each row of the projected matrix, whose
     roundings fall to both sides: sqrt(200) u on average, u = 2^-53, times three
