@@ -1029,6 +1029,28 @@ int run_variant(const Sector* s, int v, const void* x, void* y, cudaStream_t st,
 
 }  // namespace
 
+// Distinct values of one spin's hop list: T_ij times the sign of every number of
+// electrons that fits between i and j beside n - 1 others (more than kMaxCoef
+// values: any such number of them).
+static std::vector<double> hop_values(const Sector* s, int n) {
+  std::vector<double> out;
+  const int ns = s->n_s;
+  if (n < 1 || n >= ns) return out;   // no hops
+  for (int i = 0; i < ns; ++i)
+    for (int j = i + 1; j < ns; ++j) {
+      const double t = s->T[i * ns + j];
+      if (t == 0.0) continue;
+      const int between = j - i - 1, outside = ns - 2 - between;
+      const int lo = std::max(0, n - 1 - outside), hi = std::min(between, n - 1);
+      for (int k = lo; k <= std::min(hi, lo + 1); ++k) {   // two neighbouring numbers have both signs
+        const double v = (k & 1) ? -t : t;
+        if (std::find(out.begin(), out.end(), v) == out.end()) out.push_back(v);
+        if (out.size() > (size_t)kMaxCoef) return out;
+      }
+    }
+  return out;
+}
+
 int build_fast(Sector* s) {
   s->fast.ok = s->fast.gen_ok = false;
   const uint32_t D = s->dn.D;
@@ -1037,20 +1059,10 @@ int build_fast(Sector* s) {
     return ED_OK;
   if (s->dn.max_hops > 255) return ED_OK;
   if (s->dn_move && s->M * s->M > kList) return ED_OK;
-  // distinct down-hop matrix elements plus a zero used for padding
-  std::vector<double> hv(s->dn.n_hops);
-  if (s->dn.n_hops)
-    ED_TRY_CUDA(cudaMemcpy(hv.data(), s->dn.hop_val, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost));
-  std::vector<double> coef;
-  {
-    std::map<double, int> seen;
-    for (double v : hv)
-      if (!seen.count(v)) {
-        seen[v] = (int)coef.size();
-        coef.push_back(v);
-        if (coef.size() > (size_t)kMaxCoef) return ED_OK;
-      }
-  }
+  // distinct down-hop matrix elements plus a zero used for padding, from the model
+  // itself (a pass over the hop list took 0.37 of 1.2 ms at 15 sites)
+  std::vector<double> coef = hop_values(s, s->dn.n);
+  if (coef.size() > (size_t)kMaxCoef) return ED_OK;
   int zero_id = -1;
   for (size_t i = 0; i < coef.size(); ++i)
     if (coef[i] == 0.0) zero_id = (int)i;
@@ -1082,8 +1094,11 @@ int build_fast(Sector* s) {
   // windows).  So the windows start anew at each block where that pays for the
   // extra windows: N_s = 12 (8 windows either way, seven of them across blocks)
   // and 13 (15 against 14, seven across), not N_s = 15 (56 against 51).
-  std::vector<uint32_t> dbas(D), wstart;
-  ED_TRY_CUDA(cudaMemcpy(dbas.data(), s->dn.basis, sizeof(uint32_t) * D, cudaMemcpyDeviceToHost));
+  std::vector<uint32_t> dbas, wstart;
+  if (mix_delta) {
+    dbas.resize(D);
+    ED_TRY_CUDA(cudaMemcpy(dbas.data(), s->dn.basis, sizeof(uint32_t) * D, cudaMemcpyDeviceToHost));
+  }
   auto pat_of = [&](uint32_t d) { return mix_delta ? dbas[d] >> s->orb0 : 0u; };
   {
     std::vector<uint32_t> fixed, cut;
@@ -1104,16 +1119,17 @@ int build_fast(Sector* s) {
   std::vector<uint32_t> perm((size_t)n_win * kWin, D);
   std::vector<uint8_t> cnt((size_t)n_win * 4, 0);
   for (uint32_t w = 0; w < n_win; ++w) {
-    std::vector<uint32_t> ds;
-    for (uint32_t d = wstart[w]; d < wstart[w + 1]; ++d) ds.push_back(d);
-    std::stable_sort(ds.begin(), ds.end(), [&](uint32_t a, uint32_t b) {
-      return (dptr[a + 1] - dptr[a]) > (dptr[b + 1] - dptr[b]);
-    });
-    for (size_t r = 0; r < ds.size(); ++r) {
-      const uint32_t slot = (uint32_t)(r / 32), lane = (uint32_t)(r % 32);
-      perm[(size_t)w * kWin + lane * 4 + slot] = ds[r];
+    // by counting: at[c] is the place of the next string with c hops
+    const uint32_t d0 = wstart[w], d1 = wstart[w + 1];
+    uint32_t at[257] = {0};
+    for (uint32_t d = d0; d < d1; ++d) ++at[255 - (dptr[d + 1] - dptr[d]) + 1];
+    for (int c = 1; c <= 256; ++c) at[c] += at[c - 1];
+    for (uint32_t d = d0; d < d1; ++d) {
+      const uint32_t len = dptr[d + 1] - dptr[d], r = at[255 - len]++;
+      const uint32_t slot = r / 32, lane = r % 32;
+      perm[(size_t)w * kWin + lane * 4 + slot] = d;
       uint8_t& c = cnt[(size_t)w * 4 + slot];
-      c = (uint8_t)std::max<uint32_t>(c, dptr[ds[r] + 1] - dptr[ds[r]]);
+      c = (uint8_t)std::max<uint32_t>(c, len);
     }
   }
 
@@ -1132,31 +1148,36 @@ int build_fast(Sector* s) {
     for (auto& kv : m) cmask.push_back(kv.second);
   }
   const uint32_t Du = s->up.D;
-  std::vector<uint32_t> ubas(Du), rorder(Du);
-  ED_TRY_CUDA(cudaMemcpy(ubas.data(), s->up.basis, sizeof(uint32_t) * Du, cudaMemcpyDeviceToHost));
-  std::vector<uint64_t> rkey(Du, 0);
-  for (uint32_t u = 0; u < Du; ++u) {
-    uint64_t k = 0;
-    for (uint32_t mk : cmask) k = k * 33 + (uint64_t)__builtin_popcount(ubas[u] & mk);
-    rkey[u] = cmask.size() <= 12 ? k : 0;
-  }
-  std::iota(rorder.begin(), rorder.end(), 0u);
+  std::vector<uint32_t> rorder(Du);
   {
-    // inside a component, rows with equal up-hop and mixed-list lengths sit
-    // next to each other, so the two rows of a pair pad their lists little
+    // inside a component, rows with equal up-hop and mixed-list lengths (at most
+    // kList each) sit next to each other, so the two rows of a pair pad their lists
+    // little: by counting, then by component
     std::vector<uint32_t> uptr(Du + 1), mptr;
     ED_TRY_CUDA(cudaMemcpy(uptr.data(), s->up.hop_ptr, sizeof(uint32_t) * (Du + 1), cudaMemcpyDeviceToHost));
     if (s->mx_ptr) {
       mptr.resize(Du + 1);
       ED_TRY_CUDA(cudaMemcpy(mptr.data(), s->mx_ptr, sizeof(uint32_t) * (Du + 1), cudaMemcpyDeviceToHost));
     }
+    constexpr uint32_t kLens = (kList + 1) * (kList + 1);
+    std::vector<uint32_t> at(kLens + 1, 0);
     auto lens = [&](uint32_t u) {
-      return std::make_pair(uptr[u + 1] - uptr[u], mptr.empty() ? 0u : mptr[u + 1] - mptr[u]);
+      return (uptr[u + 1] - uptr[u]) * (kList + 1) + (mptr.empty() ? 0u : mptr[u + 1] - mptr[u]);
     };
-    std::stable_sort(rorder.begin(), rorder.end(), [&](uint32_t a, uint32_t b) {
-      if (rkey[a] != rkey[b]) return rkey[a] < rkey[b];
-      return lens(a) < lens(b);
-    });
+    for (uint32_t u = 0; u < Du; ++u) ++at[lens(u) + 1];
+    for (uint32_t k = 1; k <= kLens; ++k) at[k] += at[k - 1];
+    for (uint32_t u = 0; u < Du; ++u) rorder[at[lens(u)]++] = u;
+  }
+  if (cmask.size() > 1 && cmask.size() <= 12) {
+    std::vector<uint32_t> ubas(Du);
+    ED_TRY_CUDA(cudaMemcpy(ubas.data(), s->up.basis, sizeof(uint32_t) * Du, cudaMemcpyDeviceToHost));
+    std::vector<uint64_t> rkey(Du);
+    for (uint32_t u = 0; u < Du; ++u) {
+      uint64_t k = 0;
+      for (uint32_t mk : cmask) k = k * 33 + (uint64_t)__builtin_popcount(ubas[u] & mk);
+      rkey[u] = k;
+    }
+    std::stable_sort(rorder.begin(), rorder.end(), [&](uint32_t a, uint32_t b) { return rkey[a] < rkey[b]; });
   }
 
   auto& f = s->fast;
