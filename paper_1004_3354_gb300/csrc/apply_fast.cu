@@ -1051,8 +1051,11 @@ static std::vector<double> hop_values(const Sector* s, int n) {
   return out;
 }
 
-int build_fast(Sector* s) {
+// Tables of the row kernels; allow_cut: windows may start anew at impurity
+// blocks (*cut: they do).
+static int build_rows(Sector* s, bool allow_cut, bool* cut_used) {
   s->fast.ok = s->fast.gen_ok = false;
+  *cut_used = false;
   const uint32_t D = s->dn.D;
   const bool gen = s->n_chunks > 1;   // general diagonal: the one-row kernel only
   if (D < 512 || s->up.max_hops > (uint32_t)kList || s->max_mix > (uint32_t)kList)
@@ -1108,7 +1111,8 @@ int build_fast(Sector* s) {
       if (cut.empty() || d - cut.back() == kWin || pat_of(d) != pat_of(d - 1)) cut.push_back(d);
     }
     for (uint32_t w : fixed) across += pat_of(w) != pat_of(std::min(D, w + kWin) - 1) ? 1u : 0u;
-    wstart = 10 * cut.size() < 10 * fixed.size() + 4 * across ? cut : fixed;
+    *cut_used = allow_cut && cut != fixed && 10 * cut.size() < 10 * fixed.size() + 4 * across;
+    wstart = *cut_used ? cut : fixed;
   }
   const uint32_t n_win = (uint32_t)wstart.size();
   wstart.push_back(D);
@@ -1246,6 +1250,33 @@ int build_fast(Sector* s) {
   ED_TRY(build_nat(s, coef, zero_id));
   tune_apply_cached(s);  // a variant tuned earlier for this shape (any creator: ABI, server, Green's function)
   return ED_OK;
+}
+
+// Cut windows take more tables than windows of 128 strings throughout, and a general
+// cluster needs none (its generic kernels do without): where the context's budget
+// does not hold them, the sector is made without.
+int build_fast(Sector* s) {
+  const size_t mark = s->allocs.size();
+  auto undo = [&]() {
+    for (size_t i = mark; i < s->allocs.size(); ++i) {
+      dev_free(s->ctx, s->allocs[i].first, s->allocs[i].second);
+      s->table_bytes -= s->allocs[i].second;
+    }
+    s->allocs.resize(mark);
+    s->fast = Sector::Fast();
+    set_error("");
+  };
+  bool cut = false;
+  int st = build_rows(s, true, &cut);
+  if (st == ED_ERR_OOM && cut) {
+    undo();
+    st = build_rows(s, false, &cut);
+  }
+  if (st == ED_ERR_OOM && s->n_chunks > 1) {
+    undo();
+    st = ED_OK;
+  }
+  return st;
 }
 
 // Variant index: [0, 5) single-row kernel, [5, 10) two-row kernel (launch

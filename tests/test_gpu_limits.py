@@ -1,10 +1,11 @@
-"""What creating a sector costs, in time and in device memory."""
+"""Sector creation and solvers at the edge of a context's device budget, and what
+creating a sector costs."""
 import time
 
 import pytest
 
 import workloads as W
-from tests._gpu import ensure_built, torch_cuda
+from tests._gpu import empty_vec, ensure_built, rel_err, to_dev, to_host, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -12,6 +13,81 @@ pytestmark = pytest.mark.gpu
 @pytest.fixture(scope="module")
 def env():
     return ensure_built(), torch_cuda()
+
+
+def least_budget(ed, call, hi):
+    """Smallest budget (to 64 bytes) under which call(ctx) succeeds."""
+    lo = 0
+    while hi - lo > 64:
+        mid = (lo + hi) // 2
+        try:
+            ctx = ed.ed_ctx_create(0, mid)
+        except ed.EdError:
+            lo = mid
+            continue
+        try:
+            call(ctx)
+            hi = mid
+        except ed.EdError as e:
+            assert "ED_ERR_OOM" in str(e), e
+            lo = mid
+        finally:
+            ed.ed_ctx_destroy(ctx)
+    return hi
+
+
+def product(ed, torch, sec, x, prec, n):
+    y = empty_vec(n, prec, ed, torch)
+    ed.ed_apply_h(sec, to_dev(x, prec, ed, torch), y)
+    torch.cuda.synchronize()
+    return to_host(y, prec, n, ed, torch)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+def test_row_tables_never_refuse_a_general_sector(env, prec):
+    """A cluster whose interaction spans several chunks needs no row-kernel tables:
+    where they do not fit, the sector keeps the generic kernels."""
+    ed, torch = env
+    m = W.hubbard_cluster(12, tp=0.2)
+    n = W.sector_dim(12, 6, 6)
+    made = []
+
+    def create(flags):
+        def call(ctx):
+            sec = ed.ed_sector_create(ctx, m, 6, 6, prec, flags)
+            ed.ed_sector_destroy(sec)
+        return call
+    plain = least_budget(ed, create(ed.ED_SECTOR_GENERIC), 1 << 24)
+    for budget in (plain, plain + 4096, plain + 40000, 1 << 24):
+        ctx = ed.ed_ctx_create(0, budget)
+        sec = ed.ed_sector_create(ctx, m, 6, 6, prec)
+        made.append(product(ed, torch, sec, W.random_vector(n, seed=6), prec, n))
+        ed.ed_sector_destroy(sec)
+        ed.ed_ctx_destroy(ctx)
+    tol = 2.0 ** -23 if prec == "fp32" else 1e-14
+    assert max(rel_err(a, made[0]) for a in made) <= tol
+
+
+@pytest.mark.parametrize("prec,tables", [("fp64", 629140), ("df64", 1229712), ("fp32", 1119120)])
+def test_windows_cut_at_blocks_only_where_they_fit(env, prec, tables):
+    """Windows that start anew at each impurity block take more tables than windows
+    of 128 strings throughout (`tables` bytes for 13 sites); a budget for the
+    latter is enough."""
+    ed, torch = env
+    m = W.kanamori(13, seed=1)
+    n = W.sector_dim(13, 7, 6)
+    ctx = ed.ed_ctx_create(0)
+    base = ed.ed_ctx_bytes_in_use(ctx)
+    x, made = W.random_vector(n, seed=6), []
+    ed.ed_ctx_destroy(ctx)
+    for budget in (base + tables, 1 << 24):
+        ctx = ed.ed_ctx_create(0, budget)
+        sec = ed.ed_sector_create(ctx, m, 7, 6, prec)
+        made.append(product(ed, torch, sec, x, prec, n))
+        assert ed.ed_sector_get_info(sec).kernel in (2, 4)
+        ed.ed_sector_destroy(sec)
+        ed.ed_ctx_destroy(ctx)
+    assert rel_err(made[0], made[1]) <= (2.0 ** -23 if prec == "fp32" else 1e-14)
 
 
 def test_creating_a_general_sector_stays_cheap(env):
