@@ -484,7 +484,8 @@ struct Work {
   uint32_t grid;
   double* partial;  // ctx->d_red
   Coefs c;
-  double* hpart = nullptr;  // projections' partials (reorthogonalised solvers)
+  double* hpart = nullptr;  // projections' partials (reorthogonalised solvers) ...
+  int hvecs = kCgsMaxVec;   // ... of this many basis vectors at once
   int ph = 0;               // which slot of c.scale is current
 };
 
@@ -518,27 +519,21 @@ int cgs2(Work<V>& W, const V* Vb, uint64_t stride, int nvec, V* w, LzTerm<V> lz 
     k_cgs<V, true, false><<<nb, kCgsThreads, cgs_smem<V>(kn, true, false), W.st>>>(
         Vb + (uint64_t)k0 * stride, stride, kn, w, W.n, rev, W.c.h_d + k0, W.c.h_f + k0, nullptr, W.partial, none);
   };
-  if (nvec <= kCgsMaxVec) {
+  if (nvec <= W.hvecs) {
     dots(0, nvec, 0, lz);
     k_cgs<V, true, true><<<nb, kCgsThreads, cgs_smem<V>(nvec, true, true), W.st>>>(
         Vb, stride, nvec, w, W.n, 1, W.c.h_d, W.c.h_f, W.hpart, nullptr, none);
     finish(0, nvec);
     update(0, nvec, 0);
-  } else {   // a basis of more vectors than a block's shared memory serves at once: range by range
+  } else {   // more vectors than a block's shared memory, or the partials' place, serves at once: range by range
     for (int pass = 0; pass < 2; ++pass) {
-      for (int k0 = 0; k0 < nvec; k0 += kCgsMaxVec)
-        dots(k0, std::min(kCgsMaxVec, nvec - k0), 0, pass == 0 && k0 == 0 ? lz : none);
-      for (int k0 = 0; k0 < nvec; k0 += kCgsMaxVec) update(k0, std::min(kCgsMaxVec, nvec - k0), 0);
+      for (int k0 = 0; k0 < nvec; k0 += W.hvecs)
+        dots(k0, std::min(W.hvecs, nvec - k0), 0, pass == 0 && k0 == 0 ? lz : none);
+      for (int k0 = 0; k0 < nvec; k0 += W.hvecs) update(k0, std::min(W.hvecs, nvec - k0), 0);
     }
   }
   ED_LAUNCH_CHECK();
   return ED_OK;
-}
-
-// Doubles of Work::hpart for a basis of mmax + 1 vectors.
-template <class V>
-size_t cgs_part(const Ctx* c, uint64_t n, int mmax) {
-  return (size_t)std::min(mmax + 1, kCgsMaxVec) * cgs_grid<V>(c, n);
 }
 
 // H v_j with the partials of <v_j, H v_j> in W.partial; *np of them.
@@ -594,6 +589,22 @@ struct DevBuf {
     if (p) dev_free(ctx, p, bytes);
   }
 };
+
+// Room for the projections' partials of a basis of mmax + 1 vectors.  Where the
+// budget has none beside the basis, the upper half of the context's reduction
+// scratch takes those of a few vectors at a time (four sweeps instead of three).
+template <class V>
+int cgs_room(Work<V>& W, DevBuf& buf, int mmax) {
+  const size_t nb = cgs_grid<V>(W.ctx, W.n);
+  W.hvecs = kCgsMaxVec;
+  const int st = buf.alloc(W.ctx, (size_t)std::min(mmax + 1, kCgsMaxVec) * nb * sizeof(double));
+  W.hpart = static_cast<double*>(buf.p);
+  if (st != ED_ERR_OOM) return st;
+  set_error("");
+  W.hpart = W.partial + kRedSlots / 2;
+  W.hvecs = (int)std::max<size_t>(1, kRedSlots / 2 / nb);
+  return ED_OK;
+}
 
 // Carves typed arrays out of one allocation (256-byte aligned).
 struct Carve {
@@ -687,7 +698,6 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   ED_TRY(cb.alloc(ctx, coef_bytes(mmax, std::max(kk, 1))));
   V* Vbase = static_cast<V*>(vb.p);
   V* w = Vbase + (size_t)nvec_store * ld;
-  ED_TRY(hb.alloc(ctx, cgs_part<V>(ctx, n, mmax) * sizeof(double)));
   Carve cv{static_cast<char*>(cb.p)};
   Coefs c = carve_coefs(cv, mmax);
   int ldS = mmax + 1;
@@ -705,7 +715,7 @@ int lanczos_impl(Sector* s, const ed_lanczos_opts* o, double* evals, void* evecs
   if (W.grid == 0) W.grid = 1;
   W.partial = ctx->d_red;
   W.c = c;
-  W.hpart = static_cast<double*>(hb.p);
+  ED_TRY(cgs_room(W, hb, mmax));
   uint32_t vgrid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 16);
   if (vgrid == 0) vgrid = 1;
 

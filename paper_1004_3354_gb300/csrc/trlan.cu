@@ -407,8 +407,8 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   // slots padded to 32 elements, so that each starts 16-byte aligned
   const uint64_t ld = pad32(n);
   ED_TRY(vb.alloc(ctx, ((size_t)m + 2 + n_rot) * ld * eb));
-  ED_TRY(cb.alloc(ctx, coef_bytes(m, 1) + (size_t)kMaxBasis * kMaxBasis * 8 * 4 + (size_t)kMaxBasis * 8 * 16));
-  ED_TRY(hb.alloc(ctx, cgs_part<V>(ctx, n, m) * sizeof(double)));
+  // four matrices (one of kMaxBasis + 1 columns) and three vectors beside the coefficients
+  ED_TRY(cb.alloc(ctx, coef_bytes(m, 1) + (size_t)kMaxBasis * kMaxBasis * 8 * 4 + (size_t)kMaxBasis * 8 * 4));
   V* Vb = static_cast<V*>(vb.p);
   V* w = Vb + (size_t)(m + 1) * ld;
   V* T = w + ld;  // rotation target, keep vectors of n elements back to back
@@ -431,7 +431,7 @@ int trlan_impl(Sector* s, const ed_trlan_opts* o, double* evals, void* evecs, ed
   if (W.grid == 0) W.grid = 1;
   W.partial = ctx->d_red;
   W.c = c;
-  W.hpart = static_cast<double*>(hb.p);
+  ED_TRY(cgs_room(W, hb, m));
   uint32_t vgrid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)ctx->num_sms * 16);
   if (vgrid == 0) vgrid = 1;
   auto vec = [&](int j) -> V* { return Vb + (size_t)j * ld; };

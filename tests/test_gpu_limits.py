@@ -2,6 +2,7 @@
 creating a sector costs."""
 import time
 
+import numpy as np
 import pytest
 
 import workloads as W
@@ -88,6 +89,46 @@ def test_windows_cut_at_blocks_only_where_they_fit(env, prec, tables):
         ed.ed_sector_destroy(sec)
         ed.ed_ctx_destroy(ctx)
     assert rel_err(made[0], made[1]) <= (2.0 ** -23 if prec == "fp32" else 1e-14)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("solver", ["full", "restart"])
+def test_projections_need_no_room_beside_the_basis(env, solver, prec):
+    """The reorthogonalised solvers run where the sector, the basis and the
+    coefficients fit; without room for the projections' partial sums they go
+    through the basis in smaller groups."""
+    ed, torch = env
+    m = W.kanamori(11, seed=3)
+    dim, steps, k = W.sector_dim(11, 5, 6), 40, 2
+    eb = 4 if prec == "fp32" else 8
+    vec = (dim + 31) // 32 * 32 * eb
+    out = {}
+
+    def call(ctx):
+        sec = ed.ed_sector_create(ctx, m, 5, 6, prec)
+        call.held = ed.ed_ctx_bytes_in_use(ctx)
+        try:
+            if solver == "full":
+                out["ev"] = ed.ed_lanczos(sec, k=k, tol=1e-300, max_iter=steps, check_every=steps, allow_not_converged=True)[0]
+            else:
+                out["ev"] = ed.ed_lanczos_tr(sec, k=k, tol=1e-300, max_basis=steps, keep=8, max_iter=steps,
+                                             check_every=steps, allow_not_converged=True)[0]
+        finally:
+            ed.ed_sector_destroy(sec)
+    least = least_budget(ed, call, 1 << 28)
+    if solver == "full":     # 40 + 1 basis vectors, the work vector, up to 40 KB of coefficients
+        room = (steps + 2) * vec + 40000
+    else:                    # the same, 8 vectors to rotate into, four matrices of 128 rows
+        room = (steps + 2 + 8) * vec + 4 * 128 * 128 * 8 + 40000
+    assert least - call.held <= room, (least - call.held, room)
+    ctx = ed.ed_ctx_create(0, least)
+    call(ctx)
+    ed.ed_ctx_destroy(ctx)
+    tight = out["ev"]
+    ctx = ed.ed_ctx_create(0)
+    call(ctx)
+    ed.ed_ctx_destroy(ctx)
+    assert np.max(np.abs(tight - out["ev"])) <= (1e-5 if prec == "fp32" else 1e-11) * np.max(np.abs(out["ev"]))
 
 
 def test_creating_a_general_sector_stays_cheap(env):
