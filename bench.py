@@ -82,14 +82,16 @@ def workload_config(prec, dim):
 
 # Arithmetic ceiling of one H*v.  Multiply-adds per element: the off-diagonal
 # entries of the row plus two for the diagonal (e_dn + W and e_up).  A
-# double-float multiply-add counts as 12 FP32 instructions (the kernels take 11); float vectors take one FP32
-# FMA per multiply-add (natural-order kernel, float sums); FP64 rows take one
-# DFMA.  FP32 peak from the unit counts at the 2.07 GHz maximum SM clock (152
-# SMs x 128 FP32 lanes).  The FP64 peak is the measured DFMA rate on this GPU
+# double-float multiply-add is 11 FP32 instructions in the row kernels (df_mac_row):
+# "executed".  ops_per_launch and frac count 12, as figures of kernels with the
+# longer form do.  Float vectors take one FP32 FMA per multiply-add (natural-order
+# kernel, float sums); FP64 rows take one DFMA.  FP32 peak from the unit counts at
+# the 2.07 GHz maximum SM clock (152 SMs x 128 FP32 lanes).  The FP64 peak is the measured DFMA rate on this GPU
 # (a dependent-FMA probe on every SM: 0.50 T DFMA/s, about 1.6 per SM per clock),
 # since GB300's FP64 pipe does not reach a unit-count figure.
 FP32_PEAK = 152 * 128 * 2.07e9
 DFMA_PEAK = 0.50e12
+DF_COUNTED, DF_EXECUTED = 12, 11   # FP32 instructions per double-float multiply-add
 
 
 def alu_roofline(prec, dim, nnz_per_row, launch_ms):
@@ -97,9 +99,11 @@ def alu_roofline(prec, dim, nnz_per_row, launch_ms):
     if prec == "fp64":
         ops, peak, unit = macs, DFMA_PEAK, "T DFMA/s"
     else:
-        ops, peak, unit = macs * (12 if prec == "df64" else 1), FP32_PEAK, "T FP32 instructions/s"
+        ops, peak, unit = macs * (DF_COUNTED if prec == "df64" else 1), FP32_PEAK, "T FP32 instructions/s"
     achieved = ops / (launch_ms * 1e-3)
+    executed = ops * DF_EXECUTED / DF_COUNTED if prec == "df64" else ops
     return {"bound": "alu", "achieved": round(achieved / 1e12, 3), "peak": round(peak / 1e12, 3), "unit": unit,
+            "executed": {"ops_per_launch": executed, "frac": round(executed / (launch_ms * 1e-3) / peak, 4)},
             "frac": round(achieved / peak, 4), "ops_per_launch": ops, "macs_per_element": nnz_per_row + 1.0,
             "peak_source": ("measured DFMA rate (probe)" if prec == "fp64"
                             else "unit counts x 2.07 GHz maximum SM clock")}
