@@ -87,3 +87,54 @@ def test_rotations_of_the_projected_matrix_have_no_bias(env):
         ed.ed_sector_destroy(sec)
         err.append(np.linalg.norm(ev - ref) / np.linalg.norm(ref))
     assert np.mean(err) <= 3 * 200 ** 0.5 * 2.0 ** -53, err
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64"])
+def test_batched_basis_longer_than_one_launch(env, prec):
+    """2,100 steps of a batch: its projections run range by range (at most 2,048
+    vectors a launch) while a smaller sector beside it has long been exhausted.
+    Lowest values, each once, as the oracle's dense spectrum and the single-sector
+    solver give them: 1e-11 ||H|| (a few thousand roundings of 2^-46 ||H||)."""
+    ed, ctx, torch = env
+    m = W.kanamori(8, seed=22)
+    sectors = [(4, 4), (2, 1), (3, 3)]      # 4,900, 224 and 3,136 states
+    k, steps = 16, 2100
+    b = ed.ed_batch_create(ctx, m, sectors, prec)
+    try:
+        ev = ed.ed_batch_lanczos(b, len(sectors), k=k, tol=1e-300, max_iter=steps, check_every=steps,
+                                 allow_not_converged=True)[0]
+    finally:
+        ed.ed_batch_destroy(b)
+    for q, (nu, nd) in enumerate(sectors):
+        ref = np.linalg.eigvalsh(osec.build_csr(m, nu, nd).toarray())
+        assert np.all(np.abs(ev[q] - ref[:k]) <= 1e-11 * np.max(np.abs(ref))), (q, np.max(np.abs(ev[q] - ref[:k])))
+    sec = ed.ed_sector_create(ctx, m, 4, 4, prec)
+    try:
+        one, _, _ = ed.ed_lanczos(sec, k=k, tol=1e-300, max_iter=steps, check_every=steps, allow_not_converged=True)
+        assert np.all(np.abs(ev[0] - one) <= 1e-11 * np.max(np.abs(ref)))
+    finally:
+        ed.ed_sector_destroy(sec)
+
+
+@pytest.mark.parametrize("solver", ["full", "restart", "batch"])
+def test_float_projections_at_tile_edges(env, solver):
+    """Float vectors: eigenvalues to 100 u ||H|| (u = 2^-24, a few hundred roundings
+    that mostly cancel), so that an error of 1e-4 in the projections shows."""
+    ed, ctx, torch = env
+    m = W.kanamori(8, seed=21)
+    u = 2.0 ** -24
+    for nu, nd in ((1, 4), (4, 3), (4, 4)):        # 560 states (one tile and 48), 3,920, 4,900
+        ref = np.linalg.eigvalsh(osec.build_csr(m, nu, nd).toarray())
+        n, k = len(ref), 4
+        if solver == "batch":
+            b = ed.ed_batch_create(ctx, m, [(nu, nd)], "fp32")
+            ev = ed.ed_batch_lanczos(b, 1, k=k, tol=1e-5, max_iter=400, check_every=10)[0][0]
+            ed.ed_batch_destroy(b)
+        else:
+            sec = ed.ed_sector_create(ctx, m, nu, nd, "fp32")
+            if solver == "full":
+                ev, _, _ = ed.ed_lanczos(sec, k=k, tol=1e-5, max_iter=400, check_every=10)
+            else:
+                ev, _, _ = ed.ed_lanczos_tr(sec, k=k, tol=1e-5, max_basis=40, max_iter=3000)
+            ed.ed_sector_destroy(sec)
+        assert np.max(np.abs(ev - ref[:k])) <= 100 * u * np.max(np.abs(ref)), (ev, ref[:k])
