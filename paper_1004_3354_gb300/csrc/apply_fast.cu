@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
         const int c0 = c4.x, c1 = c4.y, c2 = c4.z, c3 = c4.w;
         int k = 0;
 #define ED_HOP(E, WD)                                                                     \
-  P::mac_row(acc[E], *reinterpret_cast<const C*>(reinterpret_cast<const unsigned char*>(cs) + ((WD) & 0x1fffu)), \
+  P::mac(acc[E], *reinterpret_cast<const C*>(reinterpret_cast<const unsigned char*>(cs) + ((WD) & 0x1fffu)), \
          *reinterpret_cast<const V*>(reinterpret_cast<const unsigned char*>(xs) + ((WD) >> 13)))
         for (; k < c3; ++k) {
           const uint4 h = __ldg(hp + (uint64_t)k * 32);
@@ -393,15 +393,15 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
           }
           const C c0 = lcw[k], c1 = lcw[k + 1];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) P::mac_row(acc[e], c0, a0[e]);
+          for (int e = 0; e < 4; ++e) P::mac(acc[e], c0, a0[e]);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) P::mac_row(acc[e], c1, a1[e]);
+          for (int e = 0; e < 4; ++e) P::mac(acc[e], c1, a1[e]);
         }
         if (k < nlw) {
           const V* x0 = x + lrw[k];
           const C c0 = lcw[k];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) P::mac_row(acc[e], c0, __ldg(x0 + dv[e]));
+          for (int e = 0; e < 4; ++e) P::mac(acc[e], c0, __ldg(x0 + dv[e]));
         }
       }
       // spin-flip / pair-hop in the other windows
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-              if (md[e] != INT_MIN) P::mac_row(acc[e], (md[e] & 1) ? P::neg(cj) : cj, xv[e]);
+              if (md[e] != INT_MIN) P::mac(acc[e], (md[e] & 1) ? P::neg(cj) : cj, xv[e]);
           }
         } else {
           for (int j = 0; j < nmx; ++j) {
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
             for (int e = 0; e < 4; ++e) {
               if (!ok[e]) continue;
               const int32_t mvv = __ldg(mvt + dv[e]);
-              if (mvv >= 0) P::mac_row(acc[e], (mvv & 1) ? P::neg(cj) : cj, __ldg(xm + (uint32_t)(mvv >> 1)));
+              if (mvv >= 0) P::mac(acc[e], (mvv & 1) ? P::neg(cj) : cj, __ldg(xm + (uint32_t)(mvv >> 1)));
             }
           }
         }
@@ -446,12 +446,12 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_win(FastView F, const typena
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const V xv = xs[dv[e]];
-          P::mac_row(acc[e], dg[e], xv);
-          P::mac_row(acc[e], eu, xv);
+          P::mac(acc[e], dg[e], xv);
+          P::mac(acc[e], eu, xv);
           if (GEN) {
             const uint32_t pt = sel4(gq, e);
             for (int c = 0; c < F.n_chunks; ++c)
-              P::mac_row(acc[e], ws[c * kChunkRow + ((pt >> (8 * c)) & ((1u << F.w_bits[c]) - 1u))], xv);
+              P::mac(acc[e], ws[c * kChunkRow + ((pt >> (8 * c)) & ((1u << F.w_bits[c]) - 1u))], xv);
           }
         }
       }
@@ -556,7 +556,7 @@ __device__ __forceinline__ void df_mac2s(float2& H, float2& L, float2 Ch, float2
     H = make_float2(a.x, b.x);
     L = make_float2(a.y, b.y);
   } else {
-    df_mac2<false>(H, L, Ch, Cl, Xh, Xl);
+    df_mac2(H, L, Ch, Cl, Xh);
   }
 }
 
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(BS, MINB) k_apply_pair(FastView F, const typen
         }
 #undef ED_HOP
       }
-      // the diagonal between the down and the up hops, as in the one-row kernel
+      // the diagonal between the down and the up hops
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const PV X = xs[dv[e]];

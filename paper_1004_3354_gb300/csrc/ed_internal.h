@@ -347,27 +347,17 @@ __device__ __forceinline__ void df_mac(float2& acc, float2 c, float2 x) {
   acc.y = __fadd_rn(acc.y, __fadd_rn(t, e));
 }
 
-// acc += c * x with x a plain float.
-__device__ __forceinline__ void df_mac1(float2& acc, float2 c, float x) {
-  const float p = __fmul_rn(c.x, x);
-  float e = __fmaf_rn(c.x, x, -p);
-  e = __fmaf_rn(c.y, x, e);
-  float s, t;
-  two_sum(acc.x, p, s, t);
-  acc.x = s;
-  acc.y = __fadd_rn(acc.y, __fadd_rn(t, e));
-}
-
-// The same in eleven instructions, for the row kernels of H*v, which are bound by
-// their issue.  With p = fl(c.x x.x) and s = fl(acc.x + p), Knuth's TwoSum error of
-// that sum is v + (p - bb), bb = fl(s - acc.x); the product's own error c.x x.x -
-// p joins it in one fused multiply-add, c.x x.x - bb rounded once.  The cross
-// terms c.x x.y + c.y x.x stay a chain of their own: taking them into the error's
-// chain saves one more instruction and is slower (N_s = 15 H*v: 638 us against
-// 572 us; 602 us with df_mac).  Two roundings more than df_mac: 4% more error in a
-// dot product of ten terms, 11% in a norm, so sums of other kinds keep df_mac.  In
-// H*v the diagonal after the hops gains more than that loses (norm-wise error
-// 2.5e-15 at N_s = 15, 8.8e-15 with df_mac and the diagonal first).
+// The same in eleven instructions, for H*v, whose kernels are bound by their issue.
+// With p = fl(c.x x.x) and s = fl(acc.x + p), Knuth's TwoSum error of that sum is v +
+// (p - bb), bb = fl(s - acc.x); the product's own error c.x x.x - p joins it in one
+// fused multiply-add, c.x x.x - bb rounded once.  The cross terms c.x x.y + c.y x.x
+// stay a chain of their own: taking them into the error's chain saves one more
+// instruction and is slower (N_s = 15 H*v: 638 us against 572 us; 602 us with
+// df_mac).  Two roundings more than df_mac: 4% more error in a dot product of ten
+// terms, 11% in a norm, so those sums keep df_mac.  In H*v the diagonal after the
+// hops gains more than that loses (norm-wise error against df_mac and the diagonal
+// first: 2.5e-15 and 8.8e-15 at N_s = 15, in the generic kernels 7.2e-15 and 8.7e-15
+// at N_s = 10).
 __device__ __forceinline__ void df_mac_row(float2& acc, float2 c, float2 x) {
   const float s = __fadd_rn(acc.x, __fmul_rn(c.x, x.x));
   const float nb = __fsub_rn(acc.x, s);                     // -bb
@@ -377,7 +367,10 @@ __device__ __forceinline__ void df_mac_row(float2& acc, float2 c, float2 x) {
   acc.x = s;
 }
 
-__device__ __forceinline__ void df_mac1_row(float2& acc, float2 c, float x) {
+// acc += c * x with x a plain float, in the short form: the extra rounding is lost
+// beside the vector's own (0.4% of the error of a dot product of ten floats, 1e-14
+// in all), and projections of float vectors are 5 to 10% faster than with the other.
+__device__ __forceinline__ void df_mac1(float2& acc, float2 c, float x) {
   const float s = __fadd_rn(acc.x, __fmul_rn(c.x, x));
   const float nb = __fsub_rn(acc.x, s);
   const float v = __fsub_rn(acc.x, __fadd_rn(s, nb));
@@ -387,9 +380,9 @@ __device__ __forceinline__ void df_mac1_row(float2& acc, float2 c, float x) {
 
 // Two independent double-float accumulators at once with the paired FP32
 // instructions (add/sub/mul/fma .f32x2): H = (hi0, hi1), L = (lo0, lo1) take
-// (Ch, Cl) * (Xh, Xl) lane-wise (x a plain float when XLO is false), each lane as
-// df_mac: in the shorter form of df_mac_row the product feeds only the sum and
-// gets fused into it, and the sum's error then no longer follows from TwoSum.
+// (Ch, Cl) * X lane-wise, X plain floats, with both errors on their own: in the shorter form
+// of df_mac1 the product feeds only the sum and gets fused into it, and the
+// sum's error then no longer follows from TwoSum.
 __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
   float2 d;
   asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
@@ -399,12 +392,10 @@ __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
   return d;
 }
 
-template <bool XLO>
-__device__ __forceinline__ void df_mac2(float2& H, float2& L, float2 Ch, float2 Cl, float2 Xh, float2 Xl) {
-  const float2 P = __fmul2_rn(Ch, Xh);
-  float2 E = __ffma2_rn(Ch, Xh, make_float2(-P.x, -P.y));
-  if (XLO) E = __ffma2_rn(Ch, Xl, E);
-  E = __ffma2_rn(Cl, Xh, E);
+__device__ __forceinline__ void df_mac2(float2& H, float2& L, float2 Ch, float2 Cl, float2 X) {
+  const float2 P = __fmul2_rn(Ch, X);
+  float2 E = __ffma2_rn(Ch, X, make_float2(-P.x, -P.y));
+  E = __ffma2_rn(Cl, X, E);
   const float2 S = __fadd2_rn(H, P);
   const float2 BB = f2_sub(S, H);
   const float2 T = __fadd2_rn(f2_sub(H, f2_sub(S, BB)), f2_sub(P, BB));
@@ -438,8 +429,7 @@ __host__ __device__ inline double df_to_double(float2 a) { return (double)a.x + 
 // ------------------------------------------------------ arithmetic policies
 // A policy fixes the stored element type V, the accumulator A, the matrix
 // coefficient type C (read from the double or the double-float copy of a
-// table) and how one coefficient multiplies one element (mac; mac_row in the
-// row kernels of H*v).
+// table) and how one coefficient multiplies one element in H*v.
 struct PolF64 {
   using V = double;
   using A = double;
@@ -450,7 +440,6 @@ struct PolF64 {
   __device__ static __forceinline__ const C* ld_ptr(const double* d, const float2*) { return d; }
   __device__ static __forceinline__ C neg(C c) { return -c; }
   __device__ static __forceinline__ void mac(A& a, C c, V x) { a = fma(c, x, a); }
-  __device__ static __forceinline__ void mac_row(A& a, C c, V x) { mac(a, c, x); }
   __device__ static __forceinline__ V out(A a) { return a; }
   __device__ static __forceinline__ void dot(A& a, V x, V y) { a = fma(x, y, a); }
   __device__ static __forceinline__ A warp_sum(A a) {
@@ -469,8 +458,7 @@ struct PolDF {
   __device__ static __forceinline__ C ld(const double*, const float2* f, size_t k) { return f[k]; }
   __device__ static __forceinline__ const C* ld_ptr(const double*, const float2* f) { return f; }
   __device__ static __forceinline__ C neg(C c) { return make_float2(-c.x, -c.y); }
-  __device__ static __forceinline__ void mac(A& a, C c, V x) { df_mac(a, c, x); }
-  __device__ static __forceinline__ void mac_row(A& a, C c, V x) { df_mac_row(a, c, x); }
+  __device__ static __forceinline__ void mac(A& a, C c, V x) { df_mac_row(a, c, x); }
   __device__ static __forceinline__ V out(A a) { return df_norm(a); }
   __device__ static __forceinline__ void dot(A& a, V x, V y) { df_mac(a, x, y); }
   __device__ static __forceinline__ A warp_sum(A a) {
@@ -491,7 +479,6 @@ struct PolF32 {
   __device__ static __forceinline__ const C* ld_ptr(const double*, const float2* f) { return f; }
   __device__ static __forceinline__ C neg(C c) { return make_float2(-c.x, -c.y); }
   __device__ static __forceinline__ void mac(A& a, C c, V x) { df_mac1(a, c, x); }
-  __device__ static __forceinline__ void mac_row(A& a, C c, V x) { df_mac1_row(a, c, x); }
   __device__ static __forceinline__ V out(A a) { return __fadd_rn(a.x, a.y); }
   __device__ static __forceinline__ void dot(A& a, V x, V y) { df_mac1(a, make_float2(x, 0.f), y); }
   __device__ static __forceinline__ A warp_sum(A a) {

@@ -453,14 +453,6 @@ int ritz(const Ctx* ctx, cudaStream_t st, const V* Vb, uint64_t stride, int m, c
 
 __global__ void k_step_inc(int* step) { *step += 1; }
 
-__global__ void k_copy_f64(const void* __restrict__ a, void* __restrict__ b, uint64_t bytes8) {
-  const double* s = (const double*)a;
-  double* d = (double*)b;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < bytes8;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    d[i] = s[i];
-}
-
 // ------------------------------------------------ tridiagonal eigensolver
 // Eigenpair blockIdx.x (ascending), one warp per pair.
 __global__ void __launch_bounds__(32) k_tri_pair(const double* __restrict__ a, const double* __restrict__ b, int m,

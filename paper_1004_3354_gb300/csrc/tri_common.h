@@ -44,12 +44,13 @@ __device__ __forceinline__ int tri_exp(double v) { return __double2hiint(v) & 0x
 __device__ __forceinline__ double tri_pow2_inv(int field) { return __hiloint2double(0x7fe00000 - field, 0); }
 
 // Sturm count: eigenvalues below x of the matrix with rows ab[i] = (a_i, b_i^2),
-// entries of magnitude at most about 1.  Determinants of the leading minors,
+// entries of magnitude below 2.  Determinants of the leading minors,
 // p_i = (a_i - x) p_{i-1} - b_i^2 p_{i-2}, whose sign changes count the
 // negative pivots; a pivot p_i / p_{i-1} below 2^-100 in magnitude counts as
 // -2^-100 (a change of a_i far below rounding).  Every eight rows p is brought
 // back to about 1 by an exact power of two, so that it cannot leave the range
-// of a double (a row shrinks it by at most 2^-100 and at most triples it).
+// of a double (a row shrinks it by at most 2^-100 and multiplies it by less than
+// 8: |a - x| < 4, b^2 < 4).
 __device__ inline int sturm(const double2* __restrict__ ab, int m, double x) {
   double p0 = 1.0, p1 = ab[0].x - x;
   if (tri_exp(p1) + (100 << 20) < tri_exp(p0)) p1 = -0x1p-100;
@@ -84,7 +85,7 @@ __device__ __forceinline__ double tri_warp_max(double v) {
 
 // Eigenvalue i (ascending) by 32-way multisection of the Gershgorin interval,
 // one warp per value; ab is scratch for m rows.  The matrix is scaled by an
-// exact power of two to entries of magnitude at most 1.
+// exact power of two to a largest magnitude in [1, 2).
 __device__ inline double tri_eig_one(const double* __restrict__ a, const double* __restrict__ b, int m, int i,
                                      double2* ab) {
   const int lane = threadIdx.x;
