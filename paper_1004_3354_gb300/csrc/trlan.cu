@@ -150,8 +150,8 @@ __device__ __forceinline__ void jac_rotate(T* A, T* Y, int ld, int mp, const uin
 // off-diagonals of about 1e-6 (two sweeps) to the same criterion as sweeps in
 // FP64 throughout.
 //
-// The float sweeps work on the matrix less its mean diagonal, scaled to entries of
-// at most 1: what float resolves follows the spread of the values, not how far
+// The float sweeps work on the matrix less a diagonal entry, scaled to entries of at
+// most 1: what float resolves follows the spread of the values, not how far
 // from zero they lie.
 //
 // k > 0: a convergence check whose decomposition is not used further.  It ends
@@ -202,9 +202,7 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
   for (int i = warp; i < np; i += nw)
     for (int j = lane; j < np; j += 32)
       if (j >= i) tab[i * np - i * (i - 1) / 2 + (j - i)] = (uint16_t)(i << 8 | j);
-  double mid = 0.0;
-  for (int i = tid; i < m; i += nt) mid += Ain[(size_t)i * lda + i];
-  mid = block_sum(mid) / (double)m;
+  const double mid = Ain[(size_t)(m / 2) * (lda + 1)];
   double fro = 0.0, frof = 0.0, amax = 0.0;   // Frobenius norm, and that of the shifted matrix
   for (int i = warp; i < m; i += nw)
     for (int j = lane; j < m; j += 32) {
@@ -213,8 +211,17 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
       frof += u * u;
       amax = fmax(amax, fabs(u));
     }
-  fro = block_sum(fro);
-  frof = block_sum(frof);
+  {   // both sums in one pass
+    __shared__ double2 red2[kJacThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) {
+      fro += __shfl_xor_sync(0xffffffffu, fro, o);
+      frof += __shfl_xor_sync(0xffffffffu, frof, o);
+    }
+    if (lane == 0) red2[warp] = make_double2(fro, frof);
+    __syncthreads();
+    fro = frof = 0.0;
+    for (int w = 0; w < nw; ++w) fro += red2[w].x, frof += red2[w].y;
+  }
   for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   if (lane == 0) red[warp] = amax;
   __syncthreads();
@@ -247,7 +254,7 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
     if (tid == 0) open = 0;
     __syncthreads();
     const double b = *beta;
-    const float E = (float)(3.0 * sqrt(10.0 / m) * 0x1p-24 * sqrt(frof));
+    const float E = 3.f * 0x1p-24f * sqrtf(10.f / (float)m * (float)frof);
     for (int i = tid; i < m; i += nt) {
       const float key = Af[i * ld + i];
       int at = 0;
@@ -257,7 +264,7 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
         at += (o < key || (o == key && j < i)) ? 1 : 0;
         if (j != i) {
           const float e = fabsf(Af[i * ld + j]) + E, gap = fabsf(o - key);
-          err += e < 0.5f * gap ? e / gap * fabsf(Yf[j * ld + m - 1]) : 1.f;
+          err += e < 0.5f * gap ? __fdividef(e, gap) * fabsf(Yf[j * ld + m - 1]) : 1.f;
         }
       }
       if (at < k) {
