@@ -205,12 +205,19 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
   const double mid = Ain[(size_t)(m / 2) * (lda + 1)];
   double fro = 0.0, frof = 0.0, amax = 0.0;   // Frobenius norm, and that of the shifted matrix
   for (int i = warp; i < m; i += nw)
-    for (int j = lane; j < m; j += 32) {
-      const double v = Ain[(size_t)i * lda + j], u = i == j ? v - mid : v;
-      fro += v * v;
-      frof += u * u;
-      amax = fmax(amax, fabs(u));
-    }
+    for (int j = lane; j < m; j += 32)
+      if (i != j) {
+        const double v = Ain[(size_t)i * lda + j];
+        frof += v * v;
+        amax = fmax(amax, fabs(v));
+      }
+  fro = frof;
+  for (int i = tid; i < m; i += nt) {
+    const double d = Ain[(size_t)i * (lda + 1)], u = d - mid;
+    fro += d * d;
+    frof += u * u;
+    amax = fmax(amax, fabs(u));
+  }
   {   // both sums in one pass
     __shared__ double2 red2[kJacThreads / 32];
     for (int o = 16; o > 0; o >>= 1) {
@@ -231,7 +238,9 @@ __global__ void __launch_bounds__(kJacThreads) k_sym_jacobi(const double* __rest
   const double inv = amax > 0.0 ? 1.0 / amax : 0.0;
   for (int i = warp; i < mp; i += nw)
     for (int j = lane; j < mp; j += 32) {
-      Af[i * ld + j] = (i < m && j < m) ? (float)((Ain[(size_t)i * lda + j] - (i == j ? mid : 0.0)) * inv) : 0.f;
+      double v = (i < m && j < m) ? Ain[(size_t)i * lda + j] : 0.0;
+      if (i == j && i < m) v -= mid;
+      Af[i * ld + j] = (float)(v * inv);
       Yf[i * ld + j] = i == j ? 1.f : 0.f;
     }
   __syncthreads();
