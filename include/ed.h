@@ -127,7 +127,11 @@ typedef struct ed_sector_info {
   uint64_t csr_nnz;             /* stored CSR entries (0 without ED_SECTOR_CSR) */
   uint64_t table_bytes;         /* device bytes held by the sector */
   double   nnz_per_row;         /* mean stored entries per row of H (diagonal included) */
-  int      kernel;              /* H*v kernel in use: 0 flat, 1 row-staged (general models), 2 fast row
+  int      kernel;              /* H*v kernel in use: 0 flat, 1 row-staged (models with more than eight
+                                   interacting sites: the one-row kernel with the general diagonal
+                                   for rows of 512 strings and more whose tables fit the budget; the
+                                   generic row kernel with ED_SECTOR_GENERIC or without those tables,
+                                   from rows of 1024 strings), 2 fast row
                                    kernel, 3 fast two-row kernel (DF64 when the autotuner picks
                                    it; FP32 where 4 does not apply), 4 natural-order float kernel
                                    (the FP32 default) */
@@ -290,8 +294,8 @@ typedef struct ed_tune_result {
  * bit for bit; for double-float vectors the kernels (kernel ids 2, 3, 4) sum in
  * different orders and agree to rounding; float sectors that have the
  * natural-order kernel are tuned among its variants only.
- * Sectors without the fast kernel (ED_SECTOR_GENERIC, very short rows) have
- * nothing to tune: n_candidates = 0, chosen = -1.  Allocates two vectors for
+ * Sectors without the fast kernel (ED_SECTOR_GENERIC, very short rows, models
+ * with more than eight interacting sites) have nothing to tune: n_candidates = 0, chosen = -1.  Allocates two vectors for
  * the duration of the call.  Synchronises. */
 int ed_sector_autotune(ed_sector* s, int reps, ed_tune_result* out, void* stream);
 
@@ -478,7 +482,11 @@ int ed_batch_autotune(ed_batch* b, int steps, ed_batch_tune_result* out, void* s
  *         their sectors (full CGS2 reorthogonalisation, at most 400 steps,
  *         Ritz vectors from the stored basis), then forms each request's G
  *         from its k states as above.  Packed requests do not take slots of
- *         max_active; one pack runs at a time, on a worker thread.
+ *         max_active; one pack runs at a time, on a worker thread.  Packs pay
+ *         for k > 1 where many small sectors wait together: 64 requests of N_s
+ *         6..7, k = 4, 91 solves/s in packs against 65 one by one, of N_s 8..11
+ *         50 against 46; 16 requests of N_s 8..11 41 against 49, and with k = 1
+ *         packs are slower throughout (N_s 6..7: 201 against 235).
  * A request's kernels touch only its own buffers (and, in a pack, its own
  * work items), so its result is bitwise the same alone or in a mix.  The
  * server's context must not be used from other threads while the server

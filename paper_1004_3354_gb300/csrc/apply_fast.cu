@@ -1322,7 +1322,8 @@ int fast_default_variant(const Sector* s) {
     // Four rows per block and 32 warps per SM: 512 x 2 where two such blocks
     // fit an SM (N_s = 15: 0.277 ms against 0.328 ms for two rows, 256 x 3), also
     // with fewer tiles than blocks (N_s = 12, 231 tiles: 11.6 us against 15.4 us
-    // for 1024 x 1; 124 tiles: 9.4 us against 10.6 us for two rows, 256 x 3);
+    // for 1024 x 1; 124 tiles: 9.4 us against 10.6 us for two rows, 256 x 3; 91
+    // tiles, N_s = 14 (3,7): 22.6 us against 26.6 us, AIM 20.5 us against 24.7 us);
     // else 1024 x 1 where one fits (N_s = 16: 1.31 ms against 1.63 ms for two
     // rows, 512 x 2) and the rows give every SM its block; else two rows,
     // 256 x 3 where three blocks fit, else 512 x 2.
